@@ -20,6 +20,11 @@
 
 namespace iblb {
 
+// Threads per block of the node kernels: one warp per block while the nodes
+// fill less than two warps per SM, so that the warps spread over the SMs (an
+// SM's FP64 pipe serves one warp instruction in 16 clocks), else 128.
+static int node_block(int n) { return n <= 152 * 64 ? 32 : 128; }
+
 // ------------------------------------------------------------------ A1 forces
 // 2D ring: one thread per node.
 __global__ void k_forces_ring(const double* __restrict__ q, int N, ForceParams fp,
@@ -79,7 +84,7 @@ void launch_forces(int dim, const double* q, int N, int M, const int* tri, const
                    double* normal, double* chi, int* err, cudaStream_t s)
 {
     if (dim == 2) {
-        const int b = 128, g = (N + b - 1) / b;
+        const int b = node_block(N), g = (N + b - 1) / b;
         k_forces_ring<<<g, b, 0, s>>>(q, N, fp, phi, normal, chi, err);
     } else {
         const int b = 64;
@@ -108,7 +113,7 @@ void launch_spread(int storage, int dim, const double* q, const double* phi, int
                    uint8_t* flags, uint8_t* fine, const GridParams& g, cudaStream_t s)
 {
     if (N <= 0) return;
-    const int b = 128, grid = (N + b - 1) / b;
+    const int b = node_block(N), grid = (N + b - 1) / b;
     if (storage == ST_FP64) {
         if (dim == 2) k_spread_t<2, double><<<grid, b, 0, s>>>(q, phi, N, (double*)F, flags, fine, g);
         else k_spread_t<3, double><<<grid, b, 0, s>>>(q, phi, N, (double*)F, flags, fine, g);
@@ -141,7 +146,7 @@ void launch_interp(int storage, int dim, double* q, const void* moments, int N, 
                    bool advect, const GridParams& g, cudaStream_t s)
 {
     if (N <= 0) return;
-    const int b = 128, grid = (N + b - 1) / b;
+    const int b = node_block(N), grid = (N + b - 1) / b;
     if (storage == ST_FP64) {
         if (dim == 2) k_interp_t<2, double><<<grid, b, 0, s>>>(q, (const double*)moments, N, qdot, advect, g);
         else k_interp_t<3, double><<<grid, b, 0, s>>>(q, (const double*)moments, N, qdot, advect, g);

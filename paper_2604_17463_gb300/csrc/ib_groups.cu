@@ -228,9 +228,7 @@ __device__ __forceinline__ void node_weights3(const double* __restrict__ q, int 
     for (int k = 0; k < 3; k++) {
         const double qk = q[3 * j + k];
         const double fl = floor(qk);
-        const R fr = (R)(qk - fl);
-#pragma unroll
-        for (int o = 0; o < 4; o++) w[k][o] = delta4r<R>(fr + (R)(1 - o));
+        delta4_weights<R>((R)(qk - fl), w[k]);
     }
 }
 

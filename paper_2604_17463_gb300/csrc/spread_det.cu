@@ -87,7 +87,9 @@ __global__ void k_det_bin(const DetSlot* __restrict__ slots, const int2* __restr
         const double fl = floor(qk);
         o[k] = (int)fl - 1;
         const R fr = (R)(qk - fl);  // as node_lines: FP64 split, weights in R
-        for (int s = 0; s < 4; s++) wts[(long long)it * 12 + 4 * k + s] = delta4r<R>(fr + (R)(1 - s));
+        R w4[4];
+        delta4_weights<R>(fr, w4);
+        for (int s = 0; s < 4; s++) wts[(long long)it * 12 + 4 * k + s] = w4[s];
         org[3 * it + k] = o[k];
     }
     int b[3] = {0, 0, 0};
