@@ -162,6 +162,7 @@ k_b_stream_collide(const SlotDev* __restrict__ slots, const BItem* __restrict__ 
     using L = Stencil<Q>;
     constexpr int D = L::D;
     constexpr int ILP = BIlp<Q, ST>::value;
+    constexpr int FM = force_mode<R, false>();
     const int lane = threadIdx.x & 31;
     const int nwarps = gridDim.x * (BT / 32);
     const int wid = blockIdx.x * (BT / 32) + (threadIdx.x >> 5);
@@ -321,7 +322,6 @@ k_b_stream_collide(const SlotDev* __restrict__ slots, const BItem* __restrict__ 
                         if (D == 3) F[2 * nc + cell] = 0;
                     }
                 }
-                const CellMoments<Q, R> mo = cell_moments<Q, R>(g[k], Fx, Fy, Fz, ginv);
                 R om = omega;
                 if constexpr (EXT) {
                     if (two_tau) {
@@ -330,7 +330,7 @@ k_b_stream_collide(const SlotDev* __restrict__ slots, const BItem* __restrict__ 
                             om = omega_out;
                     }
                 }
-                cell_collide<Q, R>(g[k], mo, om, Fx, Fy, Fz, gsc);
+                const CellMoments<Q, R> mo = cell_update<Q, R, FM>(g[k], band != 0, om, Fx, Fy, Fz, ginv, gsc);
                 store_cell_flat<Q, ST>(fout, nc, cell, g[k],
                                        ST == ST_FP16 ? sr_seed(step, (long long)cell) : 0u);
                 if (WRITE_ALL || band) put_moments<D, R>(mom, nc, cell, mo.drho, mo.ux, mo.uy, mo.uz);
@@ -347,6 +347,7 @@ k_b_stream_collide(const SlotDev* __restrict__ slots, const BItem* __restrict__ 
     }
 }
 
+template <bool KEEP>
 __global__ void k_b_forces_ring(const SlotDev* __restrict__ slots, const int2* __restrict__ nodes,
                                 int nnodes)
 {
@@ -354,7 +355,7 @@ __global__ void k_b_forces_ring(const SlotDev* __restrict__ slots, const int2* _
     if (t >= nnodes) return;
     const int2 nd = nodes[t];
     const SlotDev& sd = slots[nd.x];
-    ring_node_force(sd.q, sd.N, nd.y, sd.fp, sd.phi, nullptr, nullptr, sd.err);
+    ring_node_force<KEEP>(sd.q, sd.N, nd.y, sd.fp, sd.phi, nullptr, nullptr, sd.err);
 }
 
 __global__ void k_b_face_geometry(const SlotDev* __restrict__ slots,
@@ -491,7 +492,9 @@ static void launch_b_ib(int dim, int storage, int phase, const SlotDev* slots, c
     const int node_grid = (nnodes + wb - 1) / wb;  // one thread per (slot, node)
     if (phase == 0) {  // nodal forces
         if (dim == 2) {
-            k_b_forces_ring<<<(nnodes + 127) / 128, 128, 0, s>>>(slots, nodes, nnodes);
+            const int b = 64, g = (nnodes + b - 1) / b;
+            if (storage == ST_FP16) k_b_forces_ring<true><<<g, b, 0, s>>>(slots, nodes, nnodes);
+            else k_b_forces_ring<false><<<g, b, 0, s>>>(slots, nodes, nnodes);
         } else {
             if (nfaces > 0) k_b_face_geometry<<<(nfaces + 63) / 64, 64, 0, s>>>(slots, faces, nfaces);
             k_b_node_forces<<<(nnodes + 63) / 64, 64, 0, s>>>(slots, nodes, nnodes);

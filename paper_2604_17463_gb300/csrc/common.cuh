@@ -82,6 +82,7 @@ struct StreamParams {
     double body[3];        // uniform force density
     float omega_f;         // the same in FP32 (no per-thread conversion on the FP32 paths)
     float body_f[3];
+    int has_body;          // any component of the body force is not zero
     // viscosity ratio: cells outside the interface relax with omega_out
     int two_tau;
     double omega_out;
@@ -244,7 +245,7 @@ void launch_mass_partials(int Q, int storage, const void* f, const GridParams& g
 // 2D ring: one kernel; 3D mesh: per-face geometry written as one record per
 // (face, corner) at its CSR position entry_pos[3f + corner] (8 doubles per
 // record), then a per-node sum over its contiguous records (two kernels).
-void launch_forces(int dim, const double* q, int N, int M, const int* tri, const int* csr_ptr,
+void launch_forces(int storage, int dim, const double* q, int N, int M, const int* tri, const int* csr_ptr,
                    const int* entry_pos, double* entry_rec, const ForceParams& fp, double* phi,
                    double* normal, double* chi, int* err, cudaStream_t s);
 constexpr int ENTRY_RECORD_DOUBLES = 8;

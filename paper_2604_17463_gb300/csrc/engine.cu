@@ -202,7 +202,7 @@ void enqueue_classify(iblb_sim* h, cudaStream_t s)
 // cells after.
 cudaError_t launch_sc(iblb_sim* h, cudaStream_t s, bool write_all, bool bulk = false)
 {
-    uint8_t* flags = bulk ? nullptr : h->flags;
+    uint8_t* flags = (bulk || h->N == 0) ? nullptr : h->flags;  // no interface: no band
     // the step counter of the binary16 rounding follows the buffer parity
     StreamParams sp = h->sp;
     sp.rng_in = h->rng + h->cur;
@@ -237,7 +237,7 @@ void enqueue_step(iblb_sim* h, cudaStream_t s, bool write_all, bool regroup)
 {
     if (h->N > 0) {
         if (regroup) enqueue_regroup(h, s);
-        launch_forces(h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp, h->phi, nullptr,
+        launch_forces(h->storage, h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp, h->phi, nullptr,
                       nullptr, h->err, s);
         enqueue_spread(h, s);
     }
@@ -263,7 +263,7 @@ void enqueue_step_overlapped(iblb_sim* h, cudaStream_t a, cudaStream_t b, bool w
     launch_sc(h, b, write_all, true);
     cudaEventRecord(h->ev_bulk, b);
     if (regroup) enqueue_regroup(h, a);
-    launch_forces(h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp,
+    launch_forces(h->storage, h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp,
                   h->phi, nullptr, nullptr, h->err, a);
     enqueue_spread(h, a, true);
     cudaStreamWaitEvent(a, h->ev_bulk, 0);
@@ -430,7 +430,10 @@ iblb_status iblb_create(const iblb_config* cfg, void* cuda_stream, iblb_handle* 
     sp.omega = 1.0 / c.tau;
     for (int k = 0; k < 3; k++) sp.body[k] = (k < dim) ? c.body_force[k] : 0.0;
     sp.omega_f = (float)sp.omega;
-    for (int k = 0; k < 3; k++) sp.body_f[k] = (float)sp.body[k];
+    for (int k = 0; k < 3; k++) {
+        sp.body_f[k] = (float)sp.body[k];
+        if (sp.body[k] != 0.0) sp.has_body = 1;
+    }
     h->two_tau = c.tau_out != 0.0 && c.tau_out != c.tau;
     for (int k = 0; k < 3; k++) {
         sp.uw_lo[k] = c.wall_u_lo[k];
@@ -831,7 +834,7 @@ iblb_status iblb_nodal_forces(iblb_handle h, double* phi, double* normal, double
     double *dn = nullptr, *dc = nullptr;
     CK(h, cudaMalloc(&dn, nb));
     CK(h, cudaMalloc(&dc, sizeof(double) * h->N));
-    launch_forces(h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp, h->phi, dn, dc,
+    launch_forces(h->storage, h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp, h->phi, dn, dc,
                   h->err, h->stream);
     g_launches += force_kernels(h);
     cudaError_t e = cudaGetLastError();
@@ -855,7 +858,7 @@ iblb_status iblb_force_field(iblb_handle h, double* F)
     double* tmp = nullptr;
     CK(h, cudaMalloc(&tmp, sizeof(double) * h->dim * nc));
     if (h->N > 0) {
-        launch_forces(h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp, h->phi, nullptr,
+        launch_forces(h->storage, h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp, h->phi, nullptr,
                       nullptr, h->err, h->stream);
         enqueue_regroup(h, h->stream);
         enqueue_spread(h, h->stream);
@@ -994,7 +997,7 @@ iblb_status iblb_step_profiled(iblb_handle h, int n_steps, double* kernel_ms)
         const bool regroup = ib && t % 32 == 0;
         cudaEventRecord(ev[0], h->stream);
         if (ib)
-            launch_forces(h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp, h->phi,
+            launch_forces(h->storage, h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp, h->phi,
                           nullptr, nullptr, h->err, h->stream);
         cudaEventRecord(ev[1], h->stream);
         if (regroup) enqueue_regroup(h, h->stream);
@@ -1117,7 +1120,8 @@ iblb_status iblb_autotune(iblb_handle h, int trials, iblb_tuning* chosen)
     std::vector<float> best_ms(cands.size(), 1e30f);
     std::vector<char> ok(cands.size(), 1);
     apply_tuning(h, cands[0]);
-    for (int t = 0; t < 4 * trials; t++) launch_sc(h, h->stream, false);
+    const bool bulk = overlapped(h);  // the pass that the steps will run
+    for (int t = 0; t < 4 * trials; t++) launch_sc(h, h->stream, false, bulk);
     g_launches += 4 * trials;
     (void)cudaGetLastError();
     for (int pass = 0; pass < 2; pass++) {
@@ -1128,13 +1132,13 @@ iblb_status iblb_autotune(iblb_handle h, int trials, iblb_tuning* chosen)
             // trial launches read f[cur] and write the scratch buffer
             // f[cur ^ 1] only: with every band flag clear no other state is
             // touched
-            if (launch_sc(h, h->stream, false) != cudaSuccess) {  // shape not launchable here
+            if (launch_sc(h, h->stream, false, bulk) != cudaSuccess) {  // shape not launchable here
                 (void)cudaGetLastError();
                 ok[ci] = 0;
                 continue;
             }
             cudaEventRecord(e0, h->stream);
-            for (int t = 0; t < trials; t++) launch_sc(h, h->stream, false);
+            for (int t = 0; t < trials; t++) launch_sc(h, h->stream, false, bulk);
             cudaEventRecord(e1, h->stream);
             g_launches += trials + 1;
             cudaError_t e = cudaEventSynchronize(e1);

@@ -27,13 +27,14 @@ static int node_block(int n) { return n <= 152 * 64 ? 32 : 128; }
 
 // ------------------------------------------------------------------ A1 forces
 // 2D ring: one thread per node.
+template <bool KEEP>
 __global__ void k_forces_ring(const double* __restrict__ q, int N, ForceParams fp,
                               double* __restrict__ phi, double* __restrict__ nrm,
                               double* __restrict__ chi, int* err)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= N) return;
-    ring_node_force(q, N, j, fp, phi, nrm, chi, err);
+    ring_node_force<KEEP>(q, N, j, fp, phi, nrm, chi, err);
 }
 
 // 3D mesh, pass 1: one thread per face writes its three corner records.
@@ -79,13 +80,14 @@ __global__ void k_node_forces(const double* __restrict__ q, int N, const double*
     mesh_node_force(q, j, rec, csr_ptr, fp, phi, nrm, chi, err);
 }
 
-void launch_forces(int dim, const double* q, int N, int M, const int* tri, const int* csr_ptr,
+void launch_forces(int storage, int dim, const double* q, int N, int M, const int* tri, const int* csr_ptr,
                    const int* entry_pos, double* entry_rec, const ForceParams& fp, double* phi,
                    double* normal, double* chi, int* err, cudaStream_t s)
 {
     if (dim == 2) {
         const int b = node_block(N), g = (N + b - 1) / b;
-        k_forces_ring<<<g, b, 0, s>>>(q, N, fp, phi, normal, chi, err);
+        if (storage == ST_FP16) k_forces_ring<true><<<g, b, 0, s>>>(q, N, fp, phi, normal, chi, err);
+        else k_forces_ring<false><<<g, b, 0, s>>>(q, N, fp, phi, normal, chi, err);
     } else {
         const int b = 64;
         k_face_geometry<<<(M + b - 1) / b, b, 0, s>>>(q, tri, M, entry_pos, fp, entry_rec);
@@ -113,7 +115,9 @@ void launch_spread(int storage, int dim, const double* q, const double* phi, int
                    uint8_t* flags, uint8_t* fine, const GridParams& g, cudaStream_t s)
 {
     if (N <= 0) return;
-    const int b = node_block(N), grid = (N + b - 1) / b;
+    // a 2D binary16 run keeps its warps in blocks of 128: the order in which
+    // neighbouring warps' additions reach a cell is part of its trajectory
+    const int b = (dim == 2 && storage == ST_FP16) ? 128 : node_block(N), grid = (N + b - 1) / b;
     if (storage == ST_FP64) {
         if (dim == 2) k_spread_t<2, double><<<grid, b, 0, s>>>(q, phi, N, (double*)F, flags, fine, g);
         else k_spread_t<3, double><<<grid, b, 0, s>>>(q, phi, N, (double*)F, flags, fine, g);

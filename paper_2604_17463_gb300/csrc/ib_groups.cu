@@ -228,7 +228,7 @@ __device__ __forceinline__ void node_weights3(const double* __restrict__ q, int 
     for (int k = 0; k < 3; k++) {
         const double qk = q[3 * j + k];
         const double fl = floor(qk);
-        delta4_weights<R>((R)(qk - fl), w[k]);
+        delta4_weights<3, R>((R)(qk - fl), w[k]);
     }
 }
 

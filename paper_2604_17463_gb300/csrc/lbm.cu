@@ -29,7 +29,7 @@ namespace iblb {
 // band != 0: the force density of the cell is added (and cleared) and the
 // moments written.  Shared by the plain kernel and the band-cell kernel of
 // the overlapped step.
-template <int Q, int ST, bool WRITE_ALL, bool CS, bool EXT>
+template <int Q, int ST, bool WRITE_ALL, bool CS, bool EXT, bool BULK = false>
 __device__ __forceinline__ void sc_cell(const typename StorageT<ST>::S* __restrict__ fin,
                                         typename StorageT<ST>::S* __restrict__ fout,
                                         typename StorageT<ST>::R* __restrict__ mom,
@@ -134,13 +134,19 @@ __device__ __forceinline__ void sc_cell(const typename StorageT<ST>::S* __restri
             }
             const long long src = ((long long)sa * ny + sy) * nx + sx;
             if (solid) {
-                g[i] = T::load(fin, (long long)L::opp(i) * nc + cell, p.inv_scale);
+                if constexpr (ST == ST_FP32 && !EXT)
+                    g[i] = load_in_order(fin + ((long long)L::opp(i) * nc + cell));
+                else
+                    g[i] = T::load(fin, (long long)L::opp(i) * nc + cell, p.inv_scale);
                 if (EXT && p.moving) {  // moving wall: + 2 w_i (c_i . u_w) / c_s^2 (rho_w = 1)
                     const double* uw = cz > 0 ? p.uw_lo : p.uw_hi;
                     g[i] += (R)(6.0 * L::w(i) * (cx * uw[0] + cy * uw[1] + cz * uw[2]));
                 }
             } else {
-                g[i] = T::load(fin, (long long)i * nc + src, p.inv_scale);
+                if constexpr (ST == ST_FP32 && !EXT)
+                    g[i] = load_in_order(fin + ((long long)i * nc + src));
+                else
+                    g[i] = T::load(fin, (long long)i * nc + src, p.inv_scale);
             }
         }
         // FP32 copies of the parameters: no FP64 conversion per thread (the
@@ -151,28 +157,29 @@ __device__ __forceinline__ void sc_cell(const typename StorageT<ST>::S* __restri
     }
 
     if (band) take_band_force<D, R>(F, nc, cell, Fx, Fy, Fz);
-    CellMoments<Q, R> mo;
-    if constexpr (ST == ST_FP16)
-        mo = cell_moments<Q, R>(g, Fx, Fy, Fz, (R)p.inv_scale);
-    else
-        mo = cell_moments<Q, R>(g, Fx, Fy, Fz);
     R om = param_omega<R>(p);
     if (EXT && p.two_tau) {  // viscosity ratio: outside the interface relax with omega_out
         const int col = (D == 2) ? x : x + nx * y;
         if (!inside_cell(p.col_cnt, p.col_z, col, a)) om = (R)p.omega_out;
     }
-    if constexpr (ST == ST_FP16) {
-        cell_collide<Q, R>(g, mo, om, Fx, Fy, Fz, (R)p.scale);
-        if constexpr (D == 2)
+    CellMoments<Q, R> mo;
+    constexpr int FM = force_mode<R, BULK>();
+    const bool force = band || p.has_body;  // uniform in the warp
+    if constexpr (D == 2) {
+        if constexpr (ST == ST_FP16) {
+            mo = cell_moments<Q, R, !BULK>(g, Fx, Fy, Fz, (R)p.inv_scale);
+            cell_collide<Q, R, !BULK>(g, mo, om, Fx, Fy, Fz, (R)p.scale);
             store_cell32<Q, ST, CS>(fout, nc, c32, g, 1.0f, sr_seed(step, cell));
-        else
-            store_cell<Q, ST, CS>(fout, nc, cell, g, 1.0f, sr_seed(step, cell));
-    } else {
-        cell_collide<Q, R>(g, mo, om, Fx, Fy, Fz);
-        if constexpr (D == 2)
+        } else {
+            mo = cell_update<Q, R, FM>(g, force, om, Fx, Fy, Fz);
             store_cell32<Q, ST, CS>(fout, nc, c32, g, p.scale, 0u);
-        else
-            store_cell<Q, ST, CS>(fout, nc, cell, g, p.scale, 0u);
+        }
+    } else if constexpr (ST == ST_FP16) {
+        mo = cell_update<Q, R, FM>(g, force, om, Fx, Fy, Fz, (R)p.inv_scale, (R)p.scale);
+        store_cell<Q, ST, CS>(fout, nc, cell, g, 1.0f, sr_seed(step, cell));
+    } else {
+        mo = cell_update<Q, R, FM>(g, force, om, Fx, Fy, Fz);
+        store_cell<Q, ST, CS>(fout, nc, cell, g, p.scale, 0u);
     }
 
     if (WRITE_ALL || band) put_moments<D, R>(mom, nc, cell, mo.drho, mo.ux, mo.uy, mo.uz);
@@ -181,8 +188,9 @@ __device__ __forceinline__ void sc_cell(const typename StorageT<ST>::S* __restri
 
 // The plain kernel: one cell per thread, blocks of BLOCK cells along x.
 // flags == nullptr: every cell takes the body force only (the bulk pass of
-// the overlapped step; the band cells are redone by k_band_sc).
-template <int Q, int ST, bool WRITE_ALL, int BLOCK, bool CS, bool EXT = false>
+// the overlapped step; the band cells are redone by k_band_sc).  BULK: the
+// same, with no body force either.
+template <int Q, int ST, bool WRITE_ALL, int BLOCK, bool CS, bool EXT = false, bool BULK = false>
 __global__ void __launch_bounds__(BLOCK)
 k_stream_collide(const typename StorageT<ST>::S* __restrict__ fin,
                  typename StorageT<ST>::S* __restrict__ fout,
@@ -204,16 +212,21 @@ k_stream_collide(const typename StorageT<ST>::S* __restrict__ fin,
     const int lane = threadIdx.x & 31;
     const long long seg = ((long long)z * p.g.ny + y) * p.g.nseg_x + (x >> 5);
     int band = 0;
-    if (lane == 0 && flags && (x >> 5) < p.g.nseg_x) band = flags[seg];
-    band = __shfl_sync(0xffffffffu, band, 0);
+    if constexpr (!BULK) {
+        if (lane == 0 && flags && (x >> 5) < p.g.nseg_x) band = flags[seg];
+        band = __shfl_sync(0xffffffffu, band, 0);
+    }
     unsigned step = 0;
     if constexpr (ST == ST_FP16)
         step = sr_step(p.rng_in, p.rng_out,
                        blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0);
     if (x >= p.g.nx) return;
-    sc_cell<Q, ST, WRITE_ALL, CS, EXT>(fin, fout, mom, F, p, x, y, z, band, step);
+    sc_cell<Q, ST, WRITE_ALL, CS, EXT, BULK>(fin, fout, mom, F, p, x, y, z, band, step);
     if (lane == 0 && band) flags[seg] = 0;
 }
+
+// A pass in which no cell has a force: no band and no body force.
+static bool bulk_launch(const uint8_t* flags, const StreamParams& p) { return !flags && !p.has_body; }
 
 template <int Q, int ST, int BLOCK, bool CS>
 static void launch_sc_b(bool write_all, const void* fin, void* fout, void* mom, void* F,
@@ -233,7 +246,12 @@ static void launch_sc_b(bool write_all, const void* fin, void* fout, void* mom, 
     auto* b = (typename T::S*)fout;
     auto* m = (typename T::R*)mom;
     auto* f = (typename T::R*)F;
-    if (write_all)
+    if (bulk_launch(flags, p)) {
+        if (write_all)
+            k_stream_collide<Q, ST, true, BLOCK, CS, false, true><<<grid, block, 0, s>>>(a, b, m, f, flags, p);
+        else
+            k_stream_collide<Q, ST, false, BLOCK, CS, false, true><<<grid, block, 0, s>>>(a, b, m, f, flags, p);
+    } else if (write_all)
         k_stream_collide<Q, ST, true, BLOCK, CS><<<grid, block, 0, s>>>(a, b, m, f, flags, p);
     else
         k_stream_collide<Q, ST, false, BLOCK, CS><<<grid, block, 0, s>>>(a, b, m, f, flags, p);
@@ -256,7 +274,12 @@ static void launch_sc_ext(bool write_all, const void* fin, void* fout, void* mom
     auto* b = (typename T::S*)fout;
     auto* m = (typename T::R*)mom;
     auto* f = (typename T::R*)F;
-    if (write_all)
+    if (bulk_launch(flags, p)) {
+        if (write_all)
+            k_stream_collide<Q, ST, true, 128, false, true, true><<<grid, 128, 0, s>>>(a, b, m, f, flags, p);
+        else
+            k_stream_collide<Q, ST, false, 128, false, true, true><<<grid, 128, 0, s>>>(a, b, m, f, flags, p);
+    } else if (write_all)
         k_stream_collide<Q, ST, true, 128, false, true><<<grid, 128, 0, s>>>(a, b, m, f, flags, p);
     else
         k_stream_collide<Q, ST, false, 128, false, true><<<grid, 128, 0, s>>>(a, b, m, f, flags, p);
@@ -348,8 +371,11 @@ k_band_list(const uint8_t* __restrict__ flags, const uint8_t* __restrict__ fine,
         if (qm & (1u << k)) list[pos++] = (int)(4 * sg + k);
 }
 
+// Latency-bound: each warp makes one or two dependent rounds of loads, so the
+// launch bounds leave registers for all of a cell's loads in flight (binary16
+// D3Q19: 20 us per step with 79 registers, 36 us with 52).
 template <int Q, int ST, bool EXT>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, ST == ST_FP64 ? 1 : (Q == 19 ? 6 : 8))
 k_band_sc(const typename StorageT<ST>::S* __restrict__ fin,
           typename StorageT<ST>::S* __restrict__ fout, typename StorageT<ST>::R* __restrict__ mom,
           typename StorageT<ST>::R* __restrict__ F, uint8_t* __restrict__ flags,
@@ -475,7 +501,7 @@ template <> struct Pair<ST_FP16> {
     }
 };
 
-template <int Q, int ST, bool WRITE_ALL, int BLOCK>
+template <int Q, int ST, bool WRITE_ALL, int BLOCK, bool BULK>
 __global__ void __launch_bounds__(BLOCK)
 k_stream_collide2(const typename StorageT<ST>::S* __restrict__ fin,
                   typename StorageT<ST>::S* __restrict__ fout, float* __restrict__ mom,
@@ -505,9 +531,12 @@ k_stream_collide2(const typename StorageT<ST>::S* __restrict__ fin,
     const long long cell = row * nx + x0;
     // band flags: lanes 0-15 share one 32-cell segment, lanes 16-31 the next
     const long long seg = row * p.g.nseg_x + (x0 >> 5);
-    int fl = 0;
-    if ((lane & 15) == 0 && active && flags) fl = flags[seg];
-    const int band = __shfl_sync(0xffffffffu, fl, lane & 16);
+    int band = 0;
+    if constexpr (!BULK) {
+        int fl = 0;
+        if ((lane & 15) == 0 && active && flags) fl = flags[seg];
+        band = __shfl_sync(0xffffffffu, fl, lane & 16);
+    }
     unsigned step = 0;
     if constexpr (ST == ST_FP16)
         step = sr_step(p.rng_in, p.rng_out,
@@ -590,8 +619,8 @@ k_stream_collide2(const typename StorageT<ST>::S* __restrict__ fin,
         F4[cell] = make_float4(0.f, 0.f, 0.f, 0.f);
         F4[cell + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    const CellMoments2 mo = cell_moments2<Q>(g, Fx, Fy, Fz);
-    cell_collide2<Q>(g, mo, p.omega_f, Fx, Fy, Fz);
+    const CellMoments2 mo = cell_moments2<Q, !BULK>(g, Fx, Fy, Fz);
+    cell_collide2<Q, !BULK>(g, mo, p.omega_f, Fx, Fy, Fz);
     const unsigned seed = ST == ST_FP16 ? sr_seed(step, cell) : 0u;
 #pragma unroll
     for (int i = 0; i < Q; i++) P::store2(fout, (long long)i * nc + cell, g[i], p.scale, sr_bits(seed, i));
@@ -619,10 +648,15 @@ static void launch_sc2_b(bool write_all, const void* fin, void* fout, void* mom,
     }
     auto* a = (const typename T::S*)fin;
     auto* b = (typename T::S*)fout;
-    if (write_all)
-        k_stream_collide2<Q, ST, true, BLOCK><<<grid, BLOCK, 0, s>>>(a, b, (float*)mom, (float*)F, flags, p);
-    else
-        k_stream_collide2<Q, ST, false, BLOCK><<<grid, BLOCK, 0, s>>>(a, b, (float*)mom, (float*)F, flags, p);
+    auto* m = (float*)mom;
+    auto* f = (float*)F;
+    if (bulk_launch(flags, p)) {
+        if (write_all) k_stream_collide2<Q, ST, true, BLOCK, true><<<grid, BLOCK, 0, s>>>(a, b, m, f, flags, p);
+        else k_stream_collide2<Q, ST, false, BLOCK, true><<<grid, BLOCK, 0, s>>>(a, b, m, f, flags, p);
+    } else {
+        if (write_all) k_stream_collide2<Q, ST, true, BLOCK, false><<<grid, BLOCK, 0, s>>>(a, b, m, f, flags, p);
+        else k_stream_collide2<Q, ST, false, BLOCK, false><<<grid, BLOCK, 0, s>>>(a, b, m, f, flags, p);
+    }
 }
 
 template <int Q, int ST>
@@ -671,7 +705,7 @@ template <> struct RowPair<ST_FP16> {
     __device__ __forceinline__ static float load(const __half* p, unsigned i) { return __half2float(p[i]); }
 };
 
-template <int ST, bool WRITE_ALL, int BLOCK>
+template <int ST, bool WRITE_ALL, int BLOCK, bool BULK>
 __global__ void __launch_bounds__(BLOCK)
 k_stream_collide_y2(const typename StorageT<ST>::S* __restrict__ fin,
                     typename StorageT<ST>::S* __restrict__ fout, float* __restrict__ mom,
@@ -691,13 +725,16 @@ k_stream_collide_y2(const typename StorageT<ST>::S* __restrict__ fin,
     const int lane = threadIdx.x & 31;
     const unsigned rowA = (unsigned)z * (unsigned)ny + (unsigned)y0;
     const unsigned rowB = hasB ? rowA + 1u : rowA;
-    int fa = 0, fb = 0;
-    if (lane == 0 && flags && (x >> 5) < p.g.nseg_x) {
-        fa = flags[rowA * (unsigned)p.g.nseg_x + (x >> 5)];
-        fb = hasB ? flags[rowB * (unsigned)p.g.nseg_x + (x >> 5)] : 0;
+    int bandA = 0, bandB = 0;
+    if constexpr (!BULK) {
+        int fa = 0, fb = 0;
+        if (lane == 0 && flags && (x >> 5) < p.g.nseg_x) {
+            fa = flags[rowA * (unsigned)p.g.nseg_x + (x >> 5)];
+            fb = hasB ? flags[rowB * (unsigned)p.g.nseg_x + (x >> 5)] : 0;
+        }
+        bandA = __shfl_sync(0xffffffffu, fa, 0);
+        bandB = __shfl_sync(0xffffffffu, fb, 0);
     }
-    const int bandA = __shfl_sync(0xffffffffu, fa, 0);
-    const int bandB = __shfl_sync(0xffffffffu, fb, 0);
     unsigned step = 0;
     if constexpr (ST == ST_FP16)
         step = sr_step(p.rng_in, p.rng_out,
@@ -747,8 +784,8 @@ k_stream_collide_y2(const typename StorageT<ST>::S* __restrict__ fin,
     if (bandB && hasB) take_band_force<3, float>(F, nc, cellB, Fx.y, Fy.y, Fz.y);
     const float ginv = (ST == ST_FP16) ? p.inv_scale : 1.0f;
     const float gsc = (ST == ST_FP16) ? p.scale : 1.0f;
-    const CellMoments2 mo = cell_moments2<Q>(g, Fx, Fy, Fz, ginv);
-    cell_collide2<Q>(g, mo, p.omega_f, Fx, Fy, Fz, gsc);
+    const CellMoments2 mo = cell_moments2<Q, !BULK>(g, Fx, Fy, Fz, ginv);
+    cell_collide2<Q, !BULK>(g, mo, p.omega_f, Fx, Fy, Fz, gsc);
     if constexpr (ST == ST_FP16) {
         unsigned short* o = reinterpret_cast<unsigned short*>(fout);
         const unsigned seed = sr_seed(step, (long long)cellA);
@@ -787,10 +824,15 @@ static void launch_y2_b(bool write_all, const void* fin, void* fout, void* mom, 
     dim3 grid((p.g.nx + BLOCK - 1) / BLOCK, (p.g.ny + 1) / 2, p.g.nz - 2 * woff);
     auto* a = (const typename T::S*)fin;
     auto* b = (typename T::S*)fout;
-    if (write_all)
-        k_stream_collide_y2<ST, true, BLOCK><<<grid, BLOCK, 0, s>>>(a, b, (float*)mom, (float*)F, flags, p);
-    else
-        k_stream_collide_y2<ST, false, BLOCK><<<grid, BLOCK, 0, s>>>(a, b, (float*)mom, (float*)F, flags, p);
+    auto* m = (float*)mom;
+    auto* f = (float*)F;
+    if (bulk_launch(flags, p)) {
+        if (write_all) k_stream_collide_y2<ST, true, BLOCK, true><<<grid, BLOCK, 0, s>>>(a, b, m, f, flags, p);
+        else k_stream_collide_y2<ST, false, BLOCK, true><<<grid, BLOCK, 0, s>>>(a, b, m, f, flags, p);
+    } else {
+        if (write_all) k_stream_collide_y2<ST, true, BLOCK, false><<<grid, BLOCK, 0, s>>>(a, b, m, f, flags, p);
+        else k_stream_collide_y2<ST, false, BLOCK, false><<<grid, BLOCK, 0, s>>>(a, b, m, f, flags, p);
+    }
 }
 
 bool rowpair_kernel_ok(int Q, int storage, const GridParams& g)

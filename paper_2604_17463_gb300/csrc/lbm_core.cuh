@@ -14,6 +14,16 @@ namespace iblb {
 
 template <int ST> struct StorageT;
 
+// A global load that keeps its place among the others: the loads of a cell
+// are all issued before the first of them is used, whatever registers that
+// takes (the compiler otherwise sinks loads to their uses).
+__device__ __forceinline__ float load_in_order(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
 template <> struct StorageT<ST_FP64> {
     using S = double;
     using R = double;
@@ -260,43 +270,90 @@ __device__ __forceinline__ double param_body<double>(const StreamParams& p, int 
 template <>
 __device__ __forceinline__ float param_body<float>(const StreamParams& p, int k) { return p.body_f[k]; }
 
+// c_i . v with the zero components left out (0 * x and 0 + x are not folded
+// away in IEEE arithmetic: written as a plain dot product, each direction
+// would spend an instruction per zero component).
+template <int Q, typename R>
+__device__ __forceinline__ R dot_c(int i, R x, R y, R z)
+{
+    using L = Stencil<Q>;
+    const int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
+    if (cx != 0) {
+        if (cy != 0) return cx > 0 ? (cy > 0 ? x + y : x - y) : (cy > 0 ? y - x : -x - y);
+        if (cz != 0) return cx > 0 ? (cz > 0 ? x + z : x - z) : (cz > 0 ? z - x : -x - z);
+        return cx > 0 ? x : -x;
+    }
+    if (cy != 0) {
+        if (cz != 0) return cy > 0 ? (cz > 0 ? y + z : y - z) : (cz > 0 ? z - y : -y - z);
+        return cy > 0 ? y : -y;
+    }
+    return cz > 0 ? z : -z;
+}
+
 // Moments of the deviations and the velocity with the half-force term.
+// FORCE = false: the cell has no force (F = 0 gives the same values).
 template <int Q, typename R>
 struct CellMoments {
     R drho, rho, ux, uy, uz;
 };
 
-template <int Q, typename R>
+template <int Q, typename R, bool FORCE = true>
 __device__ __forceinline__ CellMoments<Q, R> cell_moments(const R* g, R Fx, R Fy, R Fz,
                                                           R ginv = R(1))
 {
     using L = Stencil<Q>;
     constexpr int D = L::D;
     R drho = 0, jx = 0, jy = 0, jz = 0;
+    if constexpr (sizeof(R) == 8) {
+        // per pair of opposite directions: one sum and one difference
+        drho = g[0];
+        bool hx = false, hy = false, hz = false;  // first term seen (folded at compile time)
 #pragma unroll
-    for (int i = 0; i < Q; i++) {
-        drho += g[i];
-        if (L::cx(i) > 0) jx += g[i];
-        if (L::cx(i) < 0) jx -= g[i];
-        if (L::cy(i) > 0) jy += g[i];
-        if (L::cy(i) < 0) jy -= g[i];
-        if (D == 3) {
-            if (L::cz(i) > 0) jz += g[i];
-            if (L::cz(i) < 0) jz -= g[i];
+        for (int i = 1; i < Q; i++) {
+            if (L::opp(i) < i) continue;
+            const int o = L::opp(i);
+            drho += g[i] + g[o];
+            const R d = g[i] - g[o];
+            if (L::cx(i)) { jx = hx ? (L::cx(i) > 0 ? jx + d : jx - d) : (L::cx(i) > 0 ? d : -d); hx = true; }
+            if (L::cy(i)) { jy = hy ? (L::cy(i) > 0 ? jy + d : jy - d) : (L::cy(i) > 0 ? d : -d); hy = true; }
+            if (D == 3 && L::cz(i)) { jz = hz ? (L::cz(i) > 0 ? jz + d : jz - d) : (L::cz(i) > 0 ? d : -d); hz = true; }
         }
+    } else {
+#pragma unroll
+        for (int i = 0; i < Q; i++) {
+            drho += g[i];
+            if (L::cx(i) > 0) jx += g[i];
+            if (L::cx(i) < 0) jx -= g[i];
+            if (L::cy(i) > 0) jy += g[i];
+            if (L::cy(i) < 0) jy -= g[i];
+            if (D == 3) {
+                if (L::cz(i) > 0) jz += g[i];
+                if (L::cz(i) < 0) jz -= g[i];
+            }
+        }
+        // g may be held scaled by a power of two (binary16 storage): ginv undoes it
+        drho *= ginv;
+        jx *= ginv;
+        jy *= ginv;
+        jz *= ginv;
     }
-    // g may be held scaled by a power of two (binary16 storage): ginv undoes it
-    drho *= ginv;
-    jx *= ginv;
-    jy *= ginv;
-    jz *= ginv;
     CellMoments<Q, R> m;
     m.drho = drho;
     m.rho = R(1) + drho;
     const R inv_rho = R(1) / m.rho;
-    m.ux = (jx + R(0.5) * Fx) * inv_rho;
-    m.uy = (jy + R(0.5) * Fy) * inv_rho;
-    m.uz = (D == 3) ? (jz + R(0.5) * Fz) * inv_rho : R(0);
+    if constexpr (FORCE && sizeof(R) == 8) {
+        m.ux = fma(R(0.5), Fx, jx) * inv_rho;
+        m.uy = fma(R(0.5), Fy, jy) * inv_rho;
+        m.uz = (D == 3) ? fma(R(0.5), Fz, jz) * inv_rho : R(0);
+    } else if constexpr (FORCE) {
+        m.ux = (jx + R(0.5) * Fx) * inv_rho;
+        m.uy = (jy + R(0.5) * Fy) * inv_rho;
+        m.uz = (D == 3) ? (jz + R(0.5) * Fz) * inv_rho : R(0);
+    } else {
+        m.ux = jx * inv_rho;
+        m.uy = jy * inv_rho;
+        m.uz = (D == 3) ? jz * inv_rho : R(0);
+    }
     return m;
 }
 
@@ -309,7 +366,20 @@ __device__ __forceinline__ CellMoments<Q, R> cell_moments(const R* g, R Fx, R Fy
 //   g*_i = (1 - omega) g_i + sym + asym,   g*_opp = (1 - omega) g_opp + sym - asym
 // with pref = 1 - omega/2; the rest direction has c = 0.  w and 3 w are
 // coef_b and coef_a (exact mass and momentum identities in FP32).
-template <int Q, typename R>
+//
+// FORCE = false drops every term in F: the kernels take it for the cells
+// outside the band when there is no body force, 97 % of a 3D drop's lattice.
+// Its values are those of FORCE = true with F = 0, bit for bit.
+// In FP64 the weights are multiplied into the cell's coefficients once per
+// speed class instead of once per direction: FP64 arithmetic bounds those
+// kernels (a warp instruction holds the SM's pipe for 16 clocks).  FP32 keeps
+// the weights outside: a coefficient a_i omega rho rounded once per cell
+// would carry a bias of the same sign into every direction and so break the
+// momentum identity of coef_a, while the products here round at random.
+// D3Q19 FP64, 160 x 160 x 96: 920 -> 566 us per launch; D2Q9 FP64,
+// 2048 x 512: 215 -> 145 us; the binary16 bulk pass of 256 x 256 x 128
+// (row pairs): 150 -> 135 us.
+template <int Q, typename R, bool FORCE = true>
 __device__ __forceinline__ void cell_collide(R* g, const CellMoments<Q, R>& m, R omega, R Fx, R Fy,
                                              R Fz, R gscale = R(1))
 {
@@ -317,28 +387,112 @@ __device__ __forceinline__ void cell_collide(R* g, const CellMoments<Q, R>& m, R
     constexpr int D = L::D;
     const R pref = R(1) - R(0.5) * omega;
     const R om1 = R(1) - omega;
-    const R uF = m.ux * Fx + m.uy * Fy + m.uz * Fz;
-    const R base = omega * (m.drho - m.rho * (R(1.5) * (m.ux * m.ux + m.uy * m.uy + m.uz * m.uz)));
-    const R sym0 = base - R(3) * pref * uF;     // common part without the (c.u) terms
-    const R k2 = omega * R(4.5) * m.rho;        // coefficient of (c.u)^2
-    const R k1 = omega * m.rho;                 // coefficient of (c.u), over 3
-    const R p9 = R(9) * pref;
-    // g held scaled by gscale (a power of two): the new terms take the same scale
-    g[0] = om1 * g[0] + (coef_b<Q, R>(0) * gscale) * sym0;
+    if constexpr (sizeof(R) == 8) {
+        // the fused multiply-adds are written out: both forms round alike
+        constexpr int AX = 1, DG = Q == 9 ? 5 : 7;  // an axis and a diagonal direction
+        R usq = fma(m.uy, m.uy, m.ux * m.ux);
+        if (D == 3) usq = fma(m.uz, m.uz, usq);
+        R sym0 = omega * fma(-m.rho, R(1.5) * usq, m.drho);  // common part without the (c.u) terms
+        if constexpr (FORCE) {
+            R uF = fma(m.uy, Fy, m.ux * Fx);
+            if (D == 3) uF = fma(m.uz, Fz, uF);
+            sym0 = fma(R(-3) * pref, uF, sym0);
+        }
+        const R k1 = omega * m.rho;
+        const R k2 = R(4.5) * k1;
+        const R ws[2] = {coef_b<Q, R>(AX) * sym0, coef_b<Q, R>(DG) * sym0};
+        const R wk[2] = {coef_b<Q, R>(AX) * k2, coef_b<Q, R>(DG) * k2};
+        const R wa[2] = {coef_a<Q, R>(AX) * k1, coef_a<Q, R>(DG) * k1};
+        const R wp[2] = {coef_b<Q, R>(AX) * (R(9) * pref), coef_b<Q, R>(DG) * (R(9) * pref)};
+        const R wf[2] = {coef_a<Q, R>(AX) * pref, coef_a<Q, R>(DG) * pref};
+        g[0] = fma(om1, g[0], coef_b<Q, R>(0) * sym0);
 #pragma unroll
-    for (int i = 1; i < Q; i++) {
-        if (L::opp(i) < i) continue;  // each pair once
-        const int o = L::opp(i);
-        const R w = coef_b<Q, R>(i) * gscale;
-        const R w3 = coef_a<Q, R>(i) * gscale;
-        const R cu = (R)L::cx(i) * m.ux + (R)L::cy(i) * m.uy + (D == 3 ? (R)L::cz(i) * m.uz : R(0));
-        const R cF = (R)L::cx(i) * Fx + (R)L::cy(i) * Fy + (D == 3 ? (R)L::cz(i) * Fz : R(0));
-        const R sym = w * (sym0 + cu * (k2 * cu + p9 * cF));
-        const R asym = w3 * (k1 * cu + pref * cF);
-        const R gi = g[i], go = g[o];
-        g[i] = om1 * gi + sym + asym;
-        g[o] = om1 * go + sym - asym;
+        for (int i = 1; i < Q; i++) {
+            if (L::opp(i) < i) continue;  // each pair once
+            const int o = L::opp(i), c = speed2<Q>(i) - 1;
+            const R cu = dot_c<Q, R>(i, m.ux, m.uy, m.uz);
+            R t = wk[c] * cu, cF = R(0);
+            if constexpr (FORCE) {
+                cF = dot_c<Q, R>(i, Fx, Fy, Fz);
+                t = fma(wp[c], cF, t);
+            }
+            const R sym = fma(cu, t, ws[c]);
+            R gi = fma(om1, g[i], sym), go = fma(om1, g[o], sym);
+            if constexpr (FORCE) {
+                gi = fma(wf[c], cF, gi);
+                go = fma(-wf[c], cF, go);
+            }
+            g[i] = fma(wa[c], cu, gi);
+            g[o] = fma(-wa[c], cu, go);
+        }
+    } else {
+        R usq = m.ux * m.ux + m.uy * m.uy;
+        if (D == 3) usq = usq + m.uz * m.uz;
+        const R base = omega * (m.drho - m.rho * (R(1.5) * usq));
+        R sym0 = base;
+        if constexpr (FORCE) {
+            R uF = m.ux * Fx + m.uy * Fy;
+            if (D == 3) uF = uF + m.uz * Fz;
+            sym0 = base - R(3) * pref * uF;
+        }
+        const R k2 = omega * R(4.5) * m.rho;        // coefficient of (c.u)^2
+        const R k1 = omega * m.rho;                 // coefficient of (c.u), over 3
+        const R p9 = R(9) * pref;
+        // g held scaled by gscale (a power of two): the new terms take the same scale
+        g[0] = om1 * g[0] + (coef_b<Q, R>(0) * gscale) * sym0;
+#pragma unroll
+        for (int i = 1; i < Q; i++) {
+            if (L::opp(i) < i) continue;  // each pair once
+            const int o = L::opp(i);
+            const R w = coef_b<Q, R>(i) * gscale;
+            const R w3 = coef_a<Q, R>(i) * gscale;
+            const R cu = dot_c<Q, R>(i, m.ux, m.uy, m.uz);
+            R sym, asym;
+            if constexpr (FORCE) {
+                const R cF = dot_c<Q, R>(i, Fx, Fy, Fz);
+                sym = w * (sym0 + cu * (k2 * cu + p9 * cF));
+                asym = w3 * (k1 * cu + pref * cF);
+            } else {
+                sym = w * (sym0 + cu * (k2 * cu));
+                asym = w3 * (k1 * cu);
+            }
+            const R gi = g[i], go = g[o];
+            g[i] = om1 * gi + sym + asym;
+            g[o] = om1 * go + sym - asym;
+        }
     }
+}
+
+// Which arithmetic a kernel carries: chosen per warp, always with the force
+// terms, or never (a bulk pass without a body force).
+enum : int { FORCE_WARP = 0, FORCE_ALWAYS = 1, FORCE_NEVER = 2 };
+
+// Moments and collision of a cell that may have a force (`force`, uniform in
+// the warp).  FP64 takes the shorter arithmetic wherever there is none.  In
+// FP32 a kernel holding both forms needs more registers and loses more by
+// that than it gains (plain D3Q19 kernel, 101 x 101 x 77: 27 us with the
+// force terms alone, 38 us with both), so there the bulk pass has its own
+// instantiation and the kernels that meet band cells always carry F.
+template <int Q, typename R, int FM>
+__device__ __forceinline__ CellMoments<Q, R> cell_update(R* g, bool force, R omega, R Fx, R Fy, R Fz,
+                                                         R ginv = R(1), R gscale = R(1))
+{
+    CellMoments<Q, R> m;
+    if (FM == FORCE_ALWAYS || (FM == FORCE_WARP && force)) {
+        m = cell_moments<Q, R, true>(g, Fx, Fy, Fz, ginv);
+        cell_collide<Q, R, true>(g, m, omega, Fx, Fy, Fz, gscale);
+    } else {
+        m = cell_moments<Q, R, false>(g, Fx, Fy, Fz, ginv);
+        cell_collide<Q, R, false>(g, m, omega, Fx, Fy, Fz, gscale);
+    }
+    return m;
+}
+
+// The arithmetic of a kernel of compute precision R; BULK: no cell has a force.
+template <typename R, bool BULK>
+__host__ __device__ constexpr int force_mode()
+{
+    return BULK ? FORCE_NEVER : (sizeof(R) == 8 ? FORCE_WARP : FORCE_ALWAYS);
 }
 
 // Band force of a cell: added to (Fx, Fy, Fz) and cleared in the buffer
@@ -395,24 +549,32 @@ struct CellMoments2 {
     float2 drho, rho, ux, uy, uz;
 };
 
-template <int Q>
+// First term of a sum or the running sum (the zero start would cost an
+// addition that IEEE arithmetic does not fold away).
+__device__ __forceinline__ float2 acc2(float2 s, float2 v, int sign, bool first)
+{
+    if (sign == 0) return s;
+    if (first) return sign > 0 ? v : sub2(p2(0.f), v);
+    return sign > 0 ? add2(s, v) : sub2(s, v);
+}
+
+template <int Q, bool FORCE = true>
 __device__ __forceinline__ CellMoments2 cell_moments2(const float2* g, float2 Fx, float2 Fy,
                                                       float2 Fz, float ginv = 1.0f)
 {
     using L = Stencil<Q>;
     constexpr int D = L::D;
     float2 drho = g[0], jx = p2(0.f), jy = p2(0.f), jz = p2(0.f);
+    bool fx = true, fy = true, fz = true;  // folded at compile time
 #pragma unroll
     for (int i = 1; i < Q; i++) {
         drho = add2(drho, g[i]);
-        if (L::cx(i) > 0) jx = add2(jx, g[i]);
-        if (L::cx(i) < 0) jx = sub2(jx, g[i]);
-        if (L::cy(i) > 0) jy = add2(jy, g[i]);
-        if (L::cy(i) < 0) jy = sub2(jy, g[i]);
-        if (D == 3) {
-            if (L::cz(i) > 0) jz = add2(jz, g[i]);
-            if (L::cz(i) < 0) jz = sub2(jz, g[i]);
-        }
+        jx = acc2(jx, g[i], L::cx(i), fx);
+        jy = acc2(jy, g[i], L::cy(i), fy);
+        if (D == 3) jz = acc2(jz, g[i], L::cz(i), fz);
+        if (L::cx(i)) fx = false;
+        if (L::cy(i)) fy = false;
+        if (L::cz(i)) fz = false;
     }
     if (ginv != 1.0f) {  // g held scaled by a power of two (binary16 storage)
         drho = mul2(drho, p2(ginv));
@@ -424,13 +586,39 @@ __device__ __forceinline__ CellMoments2 cell_moments2(const float2* g, float2 Fx
     m.drho = drho;
     m.rho = add2(p2(1.f), drho);
     const float2 inv_rho = make_float2(1.0f / m.rho.x, 1.0f / m.rho.y);
-    m.ux = mul2(fma2(p2(0.5f), Fx, jx), inv_rho);
-    m.uy = mul2(fma2(p2(0.5f), Fy, jy), inv_rho);
-    m.uz = (D == 3) ? mul2(fma2(p2(0.5f), Fz, jz), inv_rho) : p2(0.f);
+    if constexpr (FORCE) {
+        jx = fma2(p2(0.5f), Fx, jx);
+        jy = fma2(p2(0.5f), Fy, jy);
+        if (D == 3) jz = fma2(p2(0.5f), Fz, jz);
+    }
+    m.ux = mul2(jx, inv_rho);
+    m.uy = mul2(jy, inv_rho);
+    m.uz = (D == 3) ? mul2(jz, inv_rho) : p2(0.f);
     return m;
 }
 
+// c_i . v of two cells, zero components left out (see dot_c); of a pair of
+// opposite directions the one visited has a positive leading component, or
+// (-x, +y) in D2Q9.
 template <int Q>
+__device__ __forceinline__ float2 dot_c2(int i, float2 x, float2 y, float2 z)
+{
+    using L = Stencil<Q>;
+    const int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
+    if (cx > 0) {
+        if (cy != 0) return cy > 0 ? add2(x, y) : sub2(x, y);
+        if (cz != 0) return cz > 0 ? add2(x, z) : sub2(x, z);
+        return x;
+    }
+    if (cx < 0) return sub2(y, x);
+    if (cy != 0) {
+        if (cz != 0) return cz > 0 ? add2(y, z) : sub2(y, z);
+        return y;
+    }
+    return z;
+}
+
+template <int Q, bool FORCE = true>
 __device__ __forceinline__ void cell_collide2(float2* g, const CellMoments2& m, float omega,
                                               float2 Fx, float2 Fy, float2 Fz,
                                               float gscale = 1.0f)
@@ -439,10 +627,15 @@ __device__ __forceinline__ void cell_collide2(float2* g, const CellMoments2& m, 
     constexpr int D = L::D;
     const float pref = 1.0f - 0.5f * omega;
     const float2 om1 = p2(1.0f - omega);
-    const float2 uF = fma2(m.uz, Fz, fma2(m.uy, Fy, mul2(m.ux, Fx)));
-    const float2 usq = fma2(m.uz, m.uz, fma2(m.uy, m.uy, mul2(m.ux, m.ux)));
+    float2 usq = fma2(m.uy, m.uy, mul2(m.ux, m.ux));
+    if (D == 3) usq = fma2(m.uz, m.uz, usq);
     const float2 base = mul2(p2(omega), fma2(mul2(p2(-1.5f), m.rho), usq, m.drho));
-    const float2 sym0 = fma2(p2(-3.0f * pref), uF, base);
+    float2 sym0 = base;
+    if constexpr (FORCE) {
+        float2 uF = fma2(m.uy, Fy, mul2(m.ux, Fx));
+        if (D == 3) uF = fma2(m.uz, Fz, uF);
+        sym0 = fma2(p2(-3.0f * pref), uF, base);
+    }
     const float2 k2 = mul2(p2(omega * 4.5f), m.rho);
     const float2 k1 = mul2(p2(omega), m.rho);
     const float2 p1 = p2(pref), p9 = p2(9.0f * pref);
@@ -454,18 +647,15 @@ __device__ __forceinline__ void cell_collide2(float2* g, const CellMoments2& m, 
         const int o = L::opp(i);
         const float2 w = p2(coef_b<Q, float>(i) * gscale);
         const float2 w3 = p2(coef_a<Q, float>(i) * gscale);
-        float2 cu = p2(0.f), cF = p2(0.f);
-        if (L::cx(i) > 0) { cu = add2(cu, m.ux); cF = add2(cF, Fx); }
-        if (L::cx(i) < 0) { cu = sub2(cu, m.ux); cF = sub2(cF, Fx); }
-        if (L::cy(i) > 0) { cu = add2(cu, m.uy); cF = add2(cF, Fy); }
-        if (L::cy(i) < 0) { cu = sub2(cu, m.uy); cF = sub2(cF, Fy); }
-        if (D == 3) {
-            if (L::cz(i) > 0) { cu = add2(cu, m.uz); cF = add2(cF, Fz); }
-            if (L::cz(i) < 0) { cu = sub2(cu, m.uz); cF = sub2(cF, Fz); }
+        const float2 cu = dot_c2<Q>(i, m.ux, m.uy, m.uz);
+        float2 t = mul2(k2, cu), a = mul2(k1, cu);
+        if constexpr (FORCE) {
+            const float2 cF = dot_c2<Q>(i, Fx, Fy, Fz);
+            t = fma2(k2, cu, mul2(p9, cF));
+            a = fma2(k1, cu, mul2(p1, cF));
         }
-        const float2 t = fma2(k2, cu, mul2(p9, cF));
         const float2 sym = mul2(w, fma2(cu, t, sym0));
-        const float2 asym = mul2(w3, fma2(k1, cu, mul2(p1, cF)));
+        const float2 asym = mul2(w3, a);
         const float2 gi = g[i], go = g[o];
         g[i] = fma2(om1, gi, add2(sym, asym));
         g[o] = fma2(om1, go, sub2(sym, asym));

@@ -88,7 +88,7 @@ __global__ void k_det_bin(const DetSlot* __restrict__ slots, const int2* __restr
         o[k] = (int)fl - 1;
         const R fr = (R)(qk - fl);  // as node_lines: FP64 split, weights in R
         R w4[4];
-        delta4_weights<R>(fr, w4);
+        delta4_weights<D, R>(fr, w4);
         for (int s = 0; s < 4; s++) wts[(long long)it * 12 + 4 * k + s] = w4[s];
         org[3 * it + k] = o[k];
     }
