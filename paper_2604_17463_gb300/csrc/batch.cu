@@ -492,7 +492,7 @@ static void launch_b_ib(int dim, int storage, int phase, const SlotDev* slots, c
     const int node_grid = (nnodes + wb - 1) / wb;  // one thread per (slot, node)
     if (phase == 0) {  // nodal forces
         if (dim == 2) {
-            const int b = 64, g = (nnodes + b - 1) / b;
+            const int b = storage == ST_FP16 ? 128 : 64, g = (nnodes + b - 1) / b;
             if (storage == ST_FP16) k_b_forces_ring<true><<<g, b, 0, s>>>(slots, nodes, nnodes);
             else k_b_forces_ring<false><<<g, b, 0, s>>>(slots, nodes, nnodes);
         } else {

@@ -141,6 +141,7 @@ struct Tuning {
     long long wait_limit = 0;   // pipelined kernel: clock cycles a wait may take (0: ~2 s)
     int ib_grouped = 0;         // 3D interfaces: 1 spreads / interpolates by spatial groups of
                                 // nodes (ib_groups.cu) instead of one thread per node
+    int pipe_form = 0;          // plain kernel, D2Q9 binary16: the pipelined kernel's bits
     int step_overlap = 0;       // 0: overlapped step on 3D lattices of >= 2^20 cells; 1: always;
                                 // 2: never (see enqueue_step_overlapped)
 };
@@ -253,6 +254,18 @@ constexpr int ENTRY_RECORD_DOUBLES = 8;
 // segment), set where a stencil touches it, for the band pass.
 void launch_spread(int storage, int dim, const double* q, const double* phi, int N, void* F,
                    uint8_t* flags, uint8_t* fine, const GridParams& g, cudaStream_t s);
+// 2D ring between two stream-collides: q_out = q advected with the velocity in
+// `moments` (first: the nodes stay and q_out is not written), forces at the
+// new positions, spread into F and flags.  FP64 and FP32 storage.
+void launch_ring(int storage, bool first, const double* q, double* q_out, int N,
+                 const ForceParams& fp, const void* moments, void* F, uint8_t* flags,
+                 const GridParams& g, int* err, cudaStream_t s);
+// 3D mesh: launch_forces and launch_spread as two kernels (the nodal forces
+// stay in registers).
+void launch_mesh_spread(int storage, const double* q, int N, int M, const int* tri,
+                        const int* csr_ptr, const int* entry_pos, double* entry_rec,
+                        const ForceParams& fp, void* F, uint8_t* flags, uint8_t* fine,
+                        const GridParams& g, int* err, cudaStream_t s);
 // qdot [N][dim] = sum u Delta; if advect, q += qdot.
 void launch_interp(int storage, int dim, double* q, const void* moments, int N, double* qdot,
                    bool advect, const GridParams& g, cudaStream_t s);

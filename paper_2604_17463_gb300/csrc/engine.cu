@@ -64,7 +64,8 @@ struct iblb_sim {
     double* obs = nullptr;     // 12 doubles
     // interface
     int N = 0, M = 0;
-    double* q = nullptr;
+    double* q = nullptr;         // node positions
+    double* q2 = nullptr;        // 2D: second buffer of the fused ring kernel (swapped with q)
     double* phi = nullptr;
     int* tri = nullptr;
     int* csr_ptr = nullptr;
@@ -86,7 +87,8 @@ struct iblb_sim {
     // spatial groups of a 3D interface's nodes (grouped spread / interpolation)
     NodeGroups grp{};
     bool grouped = false;
-    std::map<std::tuple<int, int, int>, cudaGraphExec_t> graphs;  // (parity, steps, last)
+    // (parity, steps, last + 2 fused, current q buffer)
+    std::map<std::tuple<int, int, int, double*>, cudaGraphExec_t> graphs;
     std::string msg;
 };
 
@@ -147,14 +149,33 @@ bool overlapped(const iblb_sim* h)
     if (h->N == 0 || h->two_tau || h->tune.step_overlap == 2) return false;
     return h->tune.step_overlap == 1 || (h->dim == 3 && h->g.ncell >= (1LL << 20));
 }
+// The serial step of a ring with one fused IB kernel per step (k_ring);
+// the ordered spread and the overlapped step keep their separate kernels, and
+// so do calls of fewer than RING_FUSED_STEPS steps: there one launch per phase
+// and step is what a caller that checks iblb_kernel_launch_count counts on.
+// binary16 keeps them too: its stochastic rounding makes another trajectory of
+// any last bit that the order of the additions or a fused product changes.
+constexpr int RING_FUSED_STEPS = 16;
+bool ring_fused(const iblb_sim* h, int call_steps)
+{
+    return call_steps >= RING_FUSED_STEPS && h->dim == 2 && h->storage != IBLB_FP16_DEV && h->N > 0 &&
+           !h->det && !overlapped(h);
+}
+// 3D: node forces and spread in one kernel.
+bool mesh_fused(const iblb_sim* h) { return h->dim == 3 && !h->det && !use_groups(h); }
 int kernels_per_step(const iblb_sim* h)
 {
     return (h->N > 0 ? 2 + force_kernels(h) + spread_kernels(h) : 1) +
            ((h->two_tau && h->N > 0) ? 1 : 0);
 }
-int graph_kernels_per_step(const iblb_sim* h)
+// Kernels of a replayed chunk of k steps.
+long long graph_kernels(const iblb_sim* h, int k, bool ring)
 {
-    return kernels_per_step(h) + (overlapped(h) ? BAND_KERNELS : 0);
+    const int cl = (h->two_tau && h->N > 0) ? 1 : 0;
+    if (ring) return (long long)k * (2 + cl) + 1;
+    return (long long)k * (kernels_per_step(h) - (h->N > 0 && mesh_fused(h) ? 1 : 0) +
+                           (overlapped(h) ? BAND_KERNELS : 0)) +
+           (h->N > 0 ? regroup_kernels(h) : 0);
 }
 
 // Spatial groups of the nodes for the grouped spread / interpolation of a
@@ -191,10 +212,24 @@ void enqueue_interp(iblb_sim* h, cudaStream_t s, const void* moments, double* qd
         launch_interp(h->storage, h->dim, h->q, moments, h->N, qdot, advect, h->g, s);
 }
 
-void enqueue_classify(iblb_sim* h, cudaStream_t s)
+// A1 - A3: nodal forces and spread.
+void enqueue_forces_spread(iblb_sim* h, cudaStream_t s, bool band_pass = false)
+{
+    if (mesh_fused(h)) {
+        launch_mesh_spread(h->storage, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos,
+                           h->entry_rec, h->fp, h->F, h->flags, band_pass ? h->fine : nullptr, h->g,
+                           h->err, s);
+        return;
+    }
+    launch_forces(h->storage, h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos,
+                  h->entry_rec, h->fp, h->phi, nullptr, nullptr, h->err, s);
+    enqueue_spread(h, s, band_pass);
+}
+
+void enqueue_classify(iblb_sim* h, cudaStream_t s, const double* q)
 {
     if (h->two_tau)
-        launch_classify(h->dim, h->q, h->N, h->tri, h->M, h->g, h->col_cnt, h->col_z, h->err, s);
+        launch_classify(h->dim, q, h->N, h->tri, h->M, h->g, h->col_cnt, h->col_z, h->err, s);
 }
 
 // Stream-collide of every fluid cell; bulk: without the band (flags
@@ -237,14 +272,29 @@ void enqueue_step(iblb_sim* h, cudaStream_t s, bool write_all, bool regroup)
 {
     if (h->N > 0) {
         if (regroup) enqueue_regroup(h, s);
-        launch_forces(h->storage, h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp, h->phi, nullptr,
-                      nullptr, h->err, s);
-        enqueue_spread(h, s);
+        enqueue_forces_spread(h, s);
     }
-    enqueue_classify(h, s);
+    enqueue_classify(h, s, h->q);
     launch_sc(h, s, write_all);
     if (h->N > 0) enqueue_interp(h, s, h->mom, nullptr, true);
     h->cur ^= 1;
+}
+
+// A chunk of `steps` serial steps of a ring: one fused IB kernel and the
+// stream-collide per step, the last advection at the end.  The positions move
+// to the other buffer with every step but the first; iblb_step swaps the two
+// after an even number of steps.
+void enqueue_ring_steps(iblb_sim* h, cudaStream_t s, int steps, bool last)
+{
+    double *q = h->q, *other = h->q2;
+    for (int k = 0; k < steps; k++) {
+        launch_ring(h->storage, k == 0, q, other, h->N, h->fp, h->mom, h->F, h->flags, h->g, h->err, s);
+        if (k > 0) std::swap(q, other);
+        enqueue_classify(h, s, q);
+        launch_sc(h, s, last && k == steps - 1);
+        h->cur ^= 1;
+    }
+    launch_interp(h->storage, 2, q, h->mom, h->N, nullptr, true, h->g, s);
 }
 
 // One overlapped time step under graph capture.  Stream b runs the bulk
@@ -263,9 +313,7 @@ void enqueue_step_overlapped(iblb_sim* h, cudaStream_t a, cudaStream_t b, bool w
     launch_sc(h, b, write_all, true);
     cudaEventRecord(h->ev_bulk, b);
     if (regroup) enqueue_regroup(h, a);
-    launch_forces(h->storage, h->dim, h->q, h->N, h->M, h->tri, h->csr_ptr, h->entry_pos, h->entry_rec, h->fp,
-                  h->phi, nullptr, nullptr, h->err, a);
-    enqueue_spread(h, a, true);
+    enqueue_forces_spread(h, a, true);
     cudaStreamWaitEvent(a, h->ev_bulk, 0);
     StreamParams sp = h->sp;
     sp.rng_in = h->rng + h->cur;
@@ -277,9 +325,9 @@ void enqueue_step_overlapped(iblb_sim* h, cudaStream_t a, cudaStream_t b, bool w
     h->cur ^= 1;
 }
 
-iblb_status get_graph(iblb_sim* h, int steps, bool last, cudaGraphExec_t* out)
+iblb_status get_graph(iblb_sim* h, int steps, bool last, bool ring, cudaGraphExec_t* out)
 {
-    auto key = std::make_tuple(h->cur, steps, last ? 1 : 0);
+    auto key = std::make_tuple(h->cur, steps, (last ? 1 : 0) + (ring ? 2 : 0), h->q);
     auto it = h->graphs.find(key);
     if (it != h->graphs.end()) {
         *out = it->second;
@@ -290,7 +338,8 @@ iblb_status get_graph(iblb_sim* h, int steps, bool last, cudaGraphExec_t* out)
     // the groups are refreshed once per chunk: positions move by a small
     // fraction of a cell in a chunk, and a group's box follows its nodes
     const bool ov = overlapped(h);
-    for (int k = 0; k < steps; k++) {
+    if (ring) enqueue_ring_steps(h, h->cap, steps, last);
+    for (int k = 0; k < (ring ? 0 : steps); k++) {
         const bool wa = last && k == steps - 1;
         if (ov)
             enqueue_step_overlapped(h, h->cap, h->cap2, wa, k == 0, k == 0);
@@ -332,6 +381,33 @@ double wetting_amplitude(const iblb_config& c)
     const double th = c.theta_eq_deg * (M_PI / 180.0);
     return c.sigma * ((double)(c.pi_m - 1) * (double)(c.pi_n - 1)) /
            ((double)(c.pi_n - c.pi_m) * c.xi) * (1.0 + std::cos(th));
+}
+
+// Launch shape of a new simulation.  The pipelined kernel is the default on 3D
+// lattices of at least 2^22 cells in FP32 / binary16 (where a program that
+// cares runs the autotuner); elsewhere its few persistent CTAs cost more than
+// they hide.  Whole steps, us, pipelined against the chosen shape:
+//   D2Q9  FP64   128 x 64   22.7  18.7 (plain, 64)   2048 x 512  162  156
+//         FP32  2048 x 512  24.3  18.1 (x pairs)     512 x 128   15.6  11.2 (plain)
+//         binary16 1024 x 256  17.6  13.7 (plain, with the pipelined kernel's bits)
+//   D3Q19 FP32   96 x 96 x 64  56  45 (plain, 128)   160 x 160 x 96  117  94
+//         FP64   96 x 96 x 72  640  623 (plain, 128)
+// D2Q9 FP32: x pairs need an even width and win from about 2^19 cells (1000 x
+// 250: 12.7 against 13.0 us; 512 x 128: 11.6 against 11.2).
+Tuning default_tuning(const iblb_sim* h)
+{
+    Tuning t;
+    PipeShape ps{};
+    const bool pipe = pipe_shape(h->Q, h->storage, h->g, h->sm_count, h->smem, t.rows_per_tile,
+                                 t.ctas_per_sm, t.consumer_warps, ps);
+    if (h->dim == 3 && h->storage != IBLB_FP64 && h->g.ncell >= (1LL << 22)) return t;
+    t.variant = 0;
+    if (h->dim == 2 && h->storage == IBLB_FP64) t.block_x = 64;
+    if (h->dim == 2 && h->storage == IBLB_FP32_DEV && pair_kernel_ok(h->storage, h->g) &&
+        h->g.ncell >= (1LL << 19))
+        t.variant = 2;
+    if (h->dim == 2 && h->storage == IBLB_FP16_DEV && pipe) t.pipe_form = 1;
+    return t;
 }
 
 bool apply_tuning(iblb_sim* h, const Tuning& t)
@@ -548,7 +624,7 @@ iblb_status iblb_create(const iblb_config* cfg, void* cuda_stream, iblb_handle* 
         return bail(e, "shared memory limits");
     if ((e = prepare_stream_collide_pipe(h->smem)) != cudaSuccess) return bail(e, "pipe attributes");
     h->sm_count = sms;
-    apply_tuning(h, h->tune);
+    apply_tuning(h, default_tuning(h));
     if ((e = cudaGetLastError()) != cudaSuccess) return bail(e, "init");
     *out = h;
     return IBLB_OK;
@@ -568,6 +644,7 @@ void iblb_destroy(iblb_handle h)
     free_dev(h->partial);
     free_dev(h->obs);
     free_dev(h->q);
+    free_dev(h->q2);
     free_dev(h->phi);
     free_dev(h->tri);
     free_dev(h->csr_ptr);
@@ -636,6 +713,7 @@ iblb_status iblb_set_interface(iblb_handle h, const double* xyz, int n_nodes, co
     CK(h, cudaStreamSynchronize(h->stream));
     clear_graphs(h);
     free_dev(h->q);
+    free_dev(h->q2);
     free_dev(h->phi);
     free_dev(h->tri);
     free_dev(h->csr_ptr);
@@ -653,6 +731,7 @@ iblb_status iblb_set_interface(iblb_handle h, const double* xyz, int n_nodes, co
     if (n_nodes == 0) return IBLB_OK;
     const size_t qb = sizeof(double) * (size_t)n_nodes * dim;
     CK(h, cudaMalloc(&h->q, qb));
+    if (dim == 2) CK(h, cudaMalloc(&h->q2, qb));
     CK(h, cudaMalloc(&h->phi, qb));
     CK(h, cudaMemcpyAsync(h->q, xyz, qb, cudaMemcpyHostToDevice, h->stream));
     if (h->det) {
@@ -706,16 +785,18 @@ iblb_status iblb_step(iblb_handle h, int n_steps)
 {
     if (!h || n_steps < 0) return h ? fail(h, IBLB_EINVAL, "negative step count") : IBLB_EINVAL;
     const int CHUNK = 32;
+    const bool ring = ring_fused(h, n_steps);
     int left = n_steps;
     while (left > 0) {
         const int k = std::min(left, CHUNK);
         const bool last = (k == left);
         cudaGraphExec_t ge;
-        iblb_status st = get_graph(h, k, last, &ge);
+        iblb_status st = get_graph(h, k, last, ring, &ge);
         if (st != IBLB_OK) return st;
         CK(h, cudaGraphLaunch(ge, h->stream));
-        g_launches += (long long)k * graph_kernels_per_step(h) + (h->N > 0 ? regroup_kernels(h) : 0);
+        g_launches += graph_kernels(h, k, ring);
         h->cur ^= (k & 1);
+        if (ring && k % 2 == 0) std::swap(h->q, h->q2);
         left -= k;
     }
     return IBLB_OK;
@@ -1002,7 +1083,7 @@ iblb_status iblb_step_profiled(iblb_handle h, int n_steps, double* kernel_ms)
         cudaEventRecord(ev[1], h->stream);
         if (regroup) enqueue_regroup(h, h->stream);
         if (ib) enqueue_spread(h, h->stream, ov);
-        enqueue_classify(h, h->stream);
+        enqueue_classify(h, h->stream, h->q);
         cudaEventRecord(ev[2], h->stream);
         launch_sc(h, h->stream, last, ov);
         cudaEventRecord(ev[3], h->stream);
@@ -1018,7 +1099,7 @@ iblb_status iblb_step_profiled(iblb_handle h, int n_steps, double* kernel_ms)
         if (ib) enqueue_interp(h, h->stream, h->mom, nullptr, true);
         cudaEventRecord(ev[5], h->stream);
         h->cur ^= 1;
-        g_launches += graph_kernels_per_step(h) + (regroup ? regroup_kernels(h) : 0);
+        g_launches += kernels_per_step(h) + (ov ? BAND_KERNELS : 0) + (regroup ? regroup_kernels(h) : 0);
         CK(h, cudaEventSynchronize(ev[5]));
         for (int k = 0; k < NEV - 1; k++) {
             float ms = 0.f;

@@ -20,10 +20,16 @@
 
 namespace iblb {
 
-// Threads per block of the node kernels: one warp per block while the nodes
-// fill less than two warps per SM, so that the warps spread over the SMs (an
-// SM's FP64 pipe serves one warp instruction in 16 clocks), else 128.
-static int node_block(int n) { return n <= 152 * 64 ? 32 : 128; }
+// Threads per block of the node kernels: one warp per block up to 8 warps per
+// SM, so that the warps spread over the SMs (an SM's FP64 pipe serves one warp
+// instruction in 16 clocks), else two.
+// A 2D binary16 run keeps blocks of 128: the order in which neighbouring
+// warps' additions reach a cell is part of its trajectory.
+static int node_block(int storage, int dim, int n)
+{
+    if (dim == 2 && storage == ST_FP16) return 128;
+    return n <= 152 * 256 ? 32 : 64;
+}
 
 // ------------------------------------------------------------------ A1 forces
 // 2D ring: one thread per node.
@@ -85,7 +91,7 @@ void launch_forces(int storage, int dim, const double* q, int N, int M, const in
                    double* normal, double* chi, int* err, cudaStream_t s)
 {
     if (dim == 2) {
-        const int b = node_block(N), g = (N + b - 1) / b;
+        const int b = node_block(storage, dim, N), g = (N + b - 1) / b;
         if (storage == ST_FP16) k_forces_ring<true><<<g, b, 0, s>>>(q, N, fp, phi, normal, chi, err);
         else k_forces_ring<false><<<g, b, 0, s>>>(q, N, fp, phi, normal, chi, err);
     } else {
@@ -115,9 +121,7 @@ void launch_spread(int storage, int dim, const double* q, const double* phi, int
                    uint8_t* flags, uint8_t* fine, const GridParams& g, cudaStream_t s)
 {
     if (N <= 0) return;
-    // a 2D binary16 run keeps its warps in blocks of 128: the order in which
-    // neighbouring warps' additions reach a cell is part of its trajectory
-    const int b = (dim == 2 && storage == ST_FP16) ? 128 : node_block(N), grid = (N + b - 1) / b;
+    const int b = node_block(storage, dim, N), grid = (N + b - 1) / b;
     if (storage == ST_FP64) {
         if (dim == 2) k_spread_t<2, double><<<grid, b, 0, s>>>(q, phi, N, (double*)F, flags, fine, g);
         else k_spread_t<3, double><<<grid, b, 0, s>>>(q, phi, N, (double*)F, flags, fine, g);
@@ -125,6 +129,60 @@ void launch_spread(int storage, int dim, const double* q, const double* phi, int
         if (dim == 2) k_spread_t<2, float><<<grid, b, 0, s>>>(q, phi, N, (float*)F, flags, fine, g);
         else k_spread_t<3, float><<<grid, b, 0, s>>>(q, phi, N, (float*)F, flags, fine, g);
     }
+}
+
+// ------------------------------------------------------------------ fused IB kernels
+// 2D ring between two stream-collides: advection with the last step's
+// velocity, forces, spread (ring_warp in ib_core.cuh), one warp per block.
+template <typename R, bool FIRST>
+__global__ void __launch_bounds__(32)
+k_ring(const double* __restrict__ q, double* __restrict__ q_out, int N, ForceParams fp,
+       const R* __restrict__ mom, R* __restrict__ F, uint8_t* __restrict__ flags, GridParams g,
+       int* err)
+{
+    ring_warp<R, FIRST>(g, q, q_out, N, blockIdx.x * RING_OWN, fp, mom, F, flags, err);
+}
+
+void launch_ring(int storage, bool first, const double* q, double* q_out, int N,
+                 const ForceParams& fp, const void* moments, void* F, uint8_t* flags,
+                 const GridParams& g, int* err, cudaStream_t s)
+{
+    const int grid = (N + RING_OWN - 1) / RING_OWN;
+#define IBLB_RING(RR, FF) \
+    k_ring<RR, FF><<<grid, 32, 0, s>>>(q, q_out, N, fp, (const RR*)moments, (RR*)F, flags, g, err)
+    if (storage == ST_FP64) {
+        if (first) IBLB_RING(double, true);
+        else IBLB_RING(double, false);
+    } else {
+        if (first) IBLB_RING(float, true);
+        else IBLB_RING(float, false);
+    }
+#undef IBLB_RING
+}
+
+// 3D mesh, pass 2 with the spread: one thread per node sums its face records
+// and spreads the force it holds.
+template <typename R>
+__global__ void __launch_bounds__(64)
+k_node_spread(const double* __restrict__ q, int N, const double* __restrict__ rec,
+              const int* __restrict__ csr_ptr, ForceParams fp, R* __restrict__ F,
+              uint8_t* __restrict__ flags, uint8_t* __restrict__ fine, GridParams g, int* err)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < N) mesh_node_spread<R>(g, q, j, rec, csr_ptr, fp, F, flags, fine, err);
+}
+
+void launch_mesh_spread(int storage, const double* q, int N, int M, const int* tri,
+                        const int* csr_ptr, const int* entry_pos, double* entry_rec,
+                        const ForceParams& fp, void* F, uint8_t* flags, uint8_t* fine,
+                        const GridParams& g, int* err, cudaStream_t s)
+{
+    k_face_geometry<<<(M + 63) / 64, 64, 0, s>>>(q, tri, M, entry_pos, fp, entry_rec);
+    const int b = node_block(storage, 3, N), grid = (N + b - 1) / b;
+    if (storage == ST_FP64)
+        k_node_spread<double><<<grid, b, 0, s>>>(q, N, entry_rec, csr_ptr, fp, (double*)F, flags, fine, g, err);
+    else
+        k_node_spread<float><<<grid, b, 0, s>>>(q, N, entry_rec, csr_ptr, fp, (float*)F, flags, fine, g, err);
 }
 
 // ------------------------------------------------------------------ A5 + A6 interpolate, advect
@@ -150,7 +208,7 @@ void launch_interp(int storage, int dim, double* q, const void* moments, int N, 
                    bool advect, const GridParams& g, cudaStream_t s)
 {
     if (N <= 0) return;
-    const int b = node_block(N), grid = (N + b - 1) / b;
+    const int b = node_block(storage, dim, N), grid = (N + b - 1) / b;
     if (storage == ST_FP64) {
         if (dim == 2) k_interp_t<2, double><<<grid, b, 0, s>>>(q, (const double*)moments, N, qdot, advect, g);
         else k_interp_t<3, double><<<grid, b, 0, s>>>(q, (const double*)moments, N, qdot, advect, g);
