@@ -6,19 +6,28 @@
 // with atomics in ib.cu adds in whatever order the hardware serves them).
 //
 // Per step:
+//   0. k_det_clear   the counters (one kernel: a memset node costs a step 3 us,
+//                    a kernel 1);
 //   1. k_det_bin     per node: the 1D delta weights (as node_lines), the
 //                    stencil origin o = floor(q) - 1 per axis, the node's
 //                    bin (a tile of DT^D stencil origins), a count per bin,
 //                    and the cell tiles its stencil touches (each appended
 //                    once to a list of active cell tiles);
-//   2. k_det_scan    exclusive prefix sum of the bin counts (one block);
+//   2. k_det_scan    exclusive prefix sum of the bin counts (one block, 4096
+//                    counts at a time);
 //   3. k_det_place   node items into their bins' ranges;
 //   4. k_det_sort    each bin's items into increasing order;
-//   5. k_det_gather  per fluid cell of an active cell tile: the bins that can
-//                    hold a covering node, in a fixed order, and their nodes
-//                    in increasing order; F(x) is written (not added: the
-//                    band buffer is zero there) and the cell's band segment
-//                    flagged.
+//   5. k_det_gather  per active cell tile: the bins that can hold a node
+//                    covering one of its cells, in a fixed order, and their
+//                    nodes in increasing order, staged in shared memory with
+//                    their weights at the tile's four coordinates per axis;
+//                    every cell sums the nodes that cover it.  F(x) is written
+//                    (not added: the band buffer is zero there) and the
+//                    cell's band segment flagged.
+// The gather used to walk the bins cell by cell, matching every node's stencil
+// origin against the cell with a remainder per axis and line: 64 times the
+// index work of a node, and most of the step.  10 242 nodes on 96 x 96 x 72 in
+// FP64: spread 447 -> 128 us per step.
 // Only the order of the additions differs from the scatter: the weights are
 // the same numbers, formed the same way.  The same kernels serve the
 // single-simulation engine (one slot, node item = node id) and the batched
@@ -31,7 +40,6 @@ namespace iblb {
 namespace {
 
 constexpr int DT = DET_TILE;     // tile edge in cells (bins and cell tiles)
-constexpr int GATHER_BLOCK = 64;
 constexpr int SCAN_BLOCK = 1024;
 
 __device__ __forceinline__ int2 item_of(const int2* __restrict__ items, int it)
@@ -135,30 +143,60 @@ __global__ void k_det_bin(const DetSlot* __restrict__ slots, const int2* __restr
             }
 }
 
-// Exclusive prefix sum of cnt[0 .. n) into start and cur (one block).
+__global__ void k_det_clear(int* __restrict__ cnt, int nbins, int* __restrict__ active, int ntiles,
+                            int* __restrict__ nact)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    for (int i = t; i < nbins; i += nt) cnt[i] = 0;
+    for (int i = t; i < ntiles; i += nt) active[i] = 0;
+    if (t == 0) *nact = 0;
+}
+
+// Exclusive prefix sum of cnt[0 .. n) into start and cur (one block): 4
+// consecutive counts per thread, a scan in each warp and one over the warps.
 __global__ void __launch_bounds__(SCAN_BLOCK)
 k_det_scan(const int* __restrict__ cnt, int n, int* __restrict__ start, int* __restrict__ cur)
 {
-    __shared__ int part[SCAN_BLOCK];
-    const int t = threadIdx.x;
-    const int lo = (int)((long long)t * n / SCAN_BLOCK);
-    const int hi = (int)((long long)(t + 1) * n / SCAN_BLOCK);
-    int s = 0;
-    for (int i = lo; i < hi; i++) s += cnt[i];
-    part[t] = s;
-    __syncthreads();
-    // Hillis-Steele inclusive scan of the per-thread sums
-    for (int off = 1; off < SCAN_BLOCK; off <<= 1) {
-        const int v = t >= off ? part[t - off] : 0;
+    __shared__ int wsum[SCAN_BLOCK / 32];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    int base = 0;
+    for (int i0 = 0; i0 < n; i0 += 4 * SCAN_BLOCK) {
+        const int i = i0 + 4 * t;
+        int c[4], s = 0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            c[k] = i + k < n ? cnt[i + k] : 0;
+            s += c[k];
+        }
+        int incl = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) wsum[wid] = incl;
         __syncthreads();
-        part[t] += v;
+        if (wid == 0) {
+            int w = wsum[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, w, o);
+                if (lane >= o) w += v;
+            }
+            wsum[lane] = w;
+        }
         __syncthreads();
-    }
-    int run = part[t] - s;
-    for (int i = lo; i < hi; i++) {
-        start[i] = run;
-        cur[i] = run;
-        run += cnt[i];
+        int run = base + (wid ? wsum[wid - 1] : 0) + incl - s;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            if (i + k < n) {
+                start[i + k] = run;
+                cur[i + k] = run;
+            }
+            run += c[k];
+        }
+        base += wsum[SCAN_BLOCK / 32 - 1];
+        __syncthreads();  // wsum is written again in the next round
     }
 }
 
@@ -191,13 +229,25 @@ __global__ void k_det_sort(const int* __restrict__ cnt, const int* __restrict__ 
     }
 }
 
-// Bin tiles along axis k whose origins can cover cell coordinate x, in a
-// fixed order (origins x, x-1, x-2, x-3), without repeats.
-__device__ __forceinline__ int source_bins(const GridParams& g, int k, int x, int* out)
+// Cell coordinates of tile tc along axis k that can carry force: [lo, hi].
+__device__ __forceinline__ void tile_range(const GridParams& g, int k, int tc, int& lo, int& hi)
+{
+    const int n = extent(g, k);
+    lo = tc * DT;
+    hi = min(lo + DT, n) - 1;
+    if (!periodic_axis(g, k)) {  // fluid layers only
+        lo = max(lo, 1);
+        hi = min(hi, n - 2);
+    }
+}
+
+// Bin tiles along axis k whose origins can cover a cell of [lo, hi], in a
+// fixed order (origins hi, hi - 1, .. lo - 3), without repeats: at most 4.
+__device__ __forceinline__ int source_bins(const GridParams& g, int k, int lo, int hi, int* out)
 {
     int n = 0;
-    for (int s = 0; s < 4; s++) {
-        const int b = bin_coord(g, k, x - s) / DT;
+    for (int o = hi; o >= lo - 3; o--) {
+        const int b = bin_coord(g, k, o) / DT;
         bool seen = false;
         for (int u = 0; u < n; u++) seen |= (out[u] == b);
         if (!seen) out[n++] = b;
@@ -205,41 +255,62 @@ __device__ __forceinline__ int source_bins(const GridParams& g, int k, int x, in
     return n;
 }
 
-// Sum of the 1D weights of a node (origin o) on axis k at cell coordinate
-// x; *hit tells whether any stencil line lands on x.
+// 1D weights of a node (origin o, line weights w) on axis k at the DT
+// coordinates x0 ..; bit l of the result is set when a stencil line lands on
+// x0 + l.  On a periodic axis of fewer than 4 cells several lines land on one
+// coordinate and their weights add up.
 template <typename R>
-__device__ __forceinline__ R axis_weight(const GridParams& g, int k, int o, const R* w, int x,
-                                         bool* hit)
+__device__ __forceinline__ unsigned axis_weights(const GridParams& g, int k, int o,
+                                                 const R* __restrict__ w, int x0, R* out)
 {
-    R s = R(0);
-    bool h = false;
     const int n = extent(g, k);
     const bool per = periodic_axis(g, k);
-    for (int t = 0; t < 4; t++) {
-        const int c = per ? wrap(o + t, n) : o + t;
-        if (c == x) {
-            s = h ? s + w[t] : w[t];
-            h = true;
+    unsigned hits = 0;
+    if (per && n < 4) {
+        for (int l = 0; l < DT; l++) {
+            R s = R(0);
+            for (int t = 0; t < 4; t++)
+                if (wrap(o + t, n) == x0 + l) {
+                    s = (hits >> l) & 1u ? s + w[t] : w[t];
+                    hits |= 1u << l;
+                }
+            out[l] = s;
         }
+        return hits;
     }
-    *hit = h;
-    return s;
+    int d = per ? wrap(x0 - o, n) : x0 - o;
+#pragma unroll
+    for (int l = 0; l < DT; l++) {
+        const bool h = d >= 0 && d < 4;
+        out[l] = h ? w[d] : R(0);
+        hits |= h ? 1u << l : 0u;
+        d++;
+        if (per && d >= n) d -= n;
+    }
+    return hits;
 }
 
+// One block per active cell tile (64 threads and cells in 3D; 32 threads, 16
+// of them with a cell, in 2D); every thread stages one node of a batch.
+template <int D> constexpr int gather_block() { return D == 3 ? 64 : 32; }
+
 template <int D, typename R>
-__global__ void __launch_bounds__(GATHER_BLOCK)
+__global__ void __launch_bounds__(gather_block<D>())
 k_det_gather(const DetSlot* __restrict__ slots, const int2* __restrict__ items,
              const int2* __restrict__ act_list, const int* __restrict__ nact,
              const int* __restrict__ cnt, const int* __restrict__ start,
              const int* __restrict__ list, const int* __restrict__ org, const R* __restrict__ wts)
 {
+    constexpr int B = gather_block<D>();
     constexpr int CELLS = (D == 3) ? DT * DT * DT : DT * DT;
-    constexpr int PER = GATHER_BLOCK / CELLS;  // cell tiles per block iteration
+    constexpr int MAXBINS = (D == 3) ? 64 : 16;
+    __shared__ int s_bin[3][4], s_ns[3];
+    __shared__ int s_first[MAXBINS], s_end[MAXBINS];  // list range start, running total
+    __shared__ R s_w[B][3][DT], s_phi[B][3];
+    __shared__ unsigned s_hit[B];
+    const int t = threadIdx.x;
     const int n_act = *nact;
-    const int sub = threadIdx.x / CELLS, ci = threadIdx.x % CELLS;
-    for (int a0 = blockIdx.x * PER; a0 < n_act; a0 += gridDim.x * PER) {
-        const int a = a0 + sub;
-        if (a >= n_act) continue;
+    for (int a = blockIdx.x; a < n_act; a += gridDim.x) {
         const int2 st = act_list[a];
         const DetSlot& d = slots[st.x];
         const GridParams g = d.g;
@@ -247,41 +318,70 @@ k_det_gather(const DetSlot* __restrict__ slots, const int2* __restrict__ items,
         tc[0] = st.y % d.ct[0];
         tc[1] = (st.y / d.ct[0]) % d.ct[1];
         tc[2] = (D == 3) ? st.y / (d.ct[0] * d.ct[1]) : 0;
-        int x[3] = {tc[0] * DT + ci % DT, tc[1] * DT + (ci / DT) % DT, 0};
-        if (D == 3) x[2] = tc[2] * DT + ci / (DT * DT);
-        bool inside = true;
-        for (int k = 0; k < D; k++) {
-            const int n = extent(g, k);
-            if (x[k] >= n) inside = false;
-            if (!periodic_axis(g, k) && (x[k] < 1 || x[k] > n - 2)) inside = false;
+        __syncthreads();  // the last tile's shared arrays are read
+        if (t < 3) {
+            int nb = 1;
+            s_bin[t][0] = 0;
+            if (t < D) {
+                int lo, hi;
+                tile_range(g, t, tc[t], lo, hi);
+                nb = source_bins(g, t, lo, hi, s_bin[t]);
+            }
+            s_ns[t] = nb;
         }
-        if (!inside) continue;
-        int sb[3][4], ns[3] = {1, 1, 1};
-        sb[2][0] = 0;
-        for (int k = 0; k < D; k++) ns[k] = source_bins(g, k, x[k], sb[k]);
+        __syncthreads();
+        const int n0 = s_ns[0], n1 = s_ns[1], nbt = n0 * n1 * s_ns[2];
+        if (t < nbt) {
+            const int i0 = t % n0, i1 = (t / n0) % n1, i2 = t / (n0 * n1);
+            const int bin = d.bin_base + s_bin[0][i0] +
+                            d.nb[0] * (s_bin[1][i1] + (D == 3 ? d.nb[1] * s_bin[2][i2] : 0));
+            s_first[t] = start[bin];
+            s_end[t] = cnt[bin];
+        }
+        __syncthreads();
+        if (t == 0)
+            for (int b = 1; b < nbt; b++) s_end[b] += s_end[b - 1];
+        __syncthreads();
+        const int total = nbt > 0 ? s_end[nbt - 1] : 0;
+        const int l0 = t % DT, l1 = (t / DT) % DT, l2 = (D == 3) ? t / (DT * DT) : 0;
+        const int x[3] = {tc[0] * DT + l0, tc[1] * DT + l1, tc[2] * DT + l2};
+        bool inside = t < CELLS;
+        for (int k = 0; k < D; k++) {
+            int lo, hi;
+            tile_range(g, k, tc[k], lo, hi);
+            if (x[k] < lo || x[k] > hi) inside = false;
+        }
         R acc[3] = {R(0), R(0), R(0)};
         bool touched = false;
-        for (int i2 = 0; i2 < ns[2]; i2++)
-            for (int i1 = 0; i1 < ns[1]; i1++)
-                for (int i0 = 0; i0 < ns[0]; i0++) {
-                    const int bin = d.bin_base + sb[0][i0] +
-                                    d.nb[0] * (sb[1][i1] + (D == 3 ? d.nb[1] * sb[2][i2] : 0));
-                    const int c = cnt[bin], s0 = start[bin];
-                    for (int e = s0; e < s0 + c; e++) {
-                        const int it = list[e];
-                        const R* w = wts + (long long)it * 12;
-                        bool h0, h1, h2 = true;
-                        const R w0 = axis_weight<R>(g, 0, org[3 * it], w, x[0], &h0);
-                        const R w1 = axis_weight<R>(g, 1, org[3 * it + 1], w + 4, x[1], &h1);
-                        R w2 = R(1);
-                        if (D == 3) w2 = axis_weight<R>(g, 2, org[3 * it + 2], w + 8, x[2], &h2);
-                        if (!(h0 && h1 && h2)) continue;
-                        const R ww = (D == 3) ? w0 * w1 * w2 : w0 * w1;
-                        const int j = item_of(items, it).y;
-                        for (int k = 0; k < D; k++) acc[k] += (R)d.phi[(long long)D * j + k] * ww;
-                        touched = true;
-                    }
+        for (int e0 = 0; e0 < total; e0 += B) {
+            const int m = min(B, total - e0);
+            if (e0) __syncthreads();
+            if (t < m) {
+                const int e = e0 + t;
+                int b = 0;
+                while (e >= s_end[b]) b++;
+                const int it = list[s_first[b] + e - (b ? s_end[b - 1] : 0)];
+                const R* w = wts + (long long)it * 12;
+                unsigned hit = 0;
+#pragma unroll
+                for (int k = 0; k < D; k++)
+                    hit |= axis_weights<R>(g, k, org[3 * it + k], w + 4 * k, tc[k] * DT, s_w[t][k]) << (4 * k);
+                s_hit[t] = hit;
+                const int j = item_of(items, it).y;
+                for (int k = 0; k < D; k++) s_phi[t][k] = (R)d.phi[(long long)D * j + k];
+            }
+            __syncthreads();
+            if (inside) {
+                for (int i = 0; i < m; i++) {
+                    const unsigned hit = s_hit[i];
+                    if (!((hit >> l0) & (hit >> (4 + l1)) & (D == 3 ? hit >> (8 + l2) : 1u) & 1u)) continue;
+                    const R w01 = s_w[i][0][l0] * s_w[i][1][l1];
+                    const R ww = (D == 3) ? w01 * s_w[i][2][l2] : w01;
+                    for (int k = 0; k < D; k++) acc[k] += s_phi[i][k] * ww;
+                    touched = true;
                 }
+            }
+        }
         if (!touched) continue;
         const long long cell = ((long long)x[2] * g.ny + x[1]) * g.nx + x[0];
         R* F = (R*)d.F;
@@ -298,18 +398,17 @@ template <int D, typename R>
 void launch_det_t(const DetSlot* slots, const int2* items, int nitems, const DetBuffers& b,
                   int nbins, int ncelltiles, int sm_count, cudaStream_t s)
 {
-    cudaMemsetAsync(b.cnt, 0, sizeof(int) * (size_t)nbins, s);
-    cudaMemsetAsync(b.active, 0, sizeof(int) * (size_t)ncelltiles, s);
-    cudaMemsetAsync(b.nact, 0, sizeof(int), s);
-    const int nb = (nitems + 127) / 128;
-    k_det_bin<D, R><<<nb, 128, 0, s>>>(slots, items, nitems, b.bin_of, b.org, (R*)b.wts, b.cnt,
+    const int nclr = nbins > ncelltiles ? nbins : ncelltiles;
+    k_det_clear<<<min((nclr + 255) / 256, 4 * sm_count), 256, 0, s>>>(b.cnt, nbins, b.active,
+                                                                      ncelltiles, b.nact);
+    const int nb = (nitems + 127) / 128, nb64 = (nitems + 63) / 64;
+    k_det_bin<D, R><<<nb64, 64, 0, s>>>(slots, items, nitems, b.bin_of, b.org, (R*)b.wts, b.cnt,
                                        b.active, b.act_list, b.nact);
     k_det_scan<<<1, SCAN_BLOCK, 0, s>>>(b.cnt, nbins, b.start, b.cur);
     k_det_place<<<nb, 128, 0, s>>>(b.bin_of, nitems, b.cur, b.list);
     k_det_sort<<<(nbins + 127) / 128, 128, 0, s>>>(b.cnt, b.start, nbins, b.list);
-    k_det_gather<D, R><<<sm_count * 8, GATHER_BLOCK, 0, s>>>(slots, items, b.act_list, b.nact,
-                                                            b.cnt, b.start, b.list, b.org,
-                                                            (const R*)b.wts);
+    k_det_gather<D, R><<<sm_count * 16, gather_block<D>(), 0, s>>>(
+        slots, items, b.act_list, b.nact, b.cnt, b.start, b.list, b.org, (const R*)b.wts);
 }
 
 }  // namespace

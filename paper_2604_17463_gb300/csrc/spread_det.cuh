@@ -46,6 +46,6 @@ void launch_spread_det(int storage, int dim, const DetSlot* slots, const int2* i
                        cudaStream_t s);
 
 // Kernel launches of one deterministic spread.
-constexpr int DET_KERNELS = 5;
+constexpr int DET_KERNELS = 6;
 
 }  // namespace iblb
