@@ -307,8 +307,7 @@ typedef struct {
                                      updates the cells of the flagged band
                                      segments again, from the same sources,
                                      with their force density (the same
-                                     arithmetic as one pass).  Not used with
-                                     a viscosity ratio, nor by
+                                     arithmetic as one pass).  Not used by
                                      iblb_step_profiled.  Not changed by
                                      iblb_autotune. */
 } iblb_tuning;

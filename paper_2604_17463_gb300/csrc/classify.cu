@@ -57,11 +57,15 @@ __global__ void k_inside_mask(GridParams g, const int* __restrict__ cnt,
 
 }  // namespace
 
+void launch_classify_clear(const GridParams& g, int* cnt, cudaStream_t s)
+{
+    const size_t ncol = g.dim == 2 ? (size_t)g.nx : (size_t)g.nx * g.ny;
+    cudaMemsetAsync(cnt, 0, sizeof(int) * ncol, s);
+}
+
 void launch_classify(int dim, const double* q, int N, const int* tri, int M, const GridParams& g,
                      int* cnt, double* cz, int* err, cudaStream_t s)
 {
-    const int ncol = dim == 2 ? g.nx : g.nx * g.ny;
-    cudaMemsetAsync(cnt, 0, sizeof(int) * (size_t)ncol, s);
     if (N == 0) return;
     if (dim == 2)
         k_classify_ring<<<(N + 127) / 128, 128, 0, s>>>(q, N, g, cnt, cz, err);

@@ -205,16 +205,17 @@ cudaError_t launch_stream_collide_pipe(int Q, int storage, bool write_all, const
                                        void* fout, void* moments, void* F, uint8_t* flags,
                                        const StreamParams& p, const PipeShape& ps, cudaStream_t s);
 
-// Band cells of the overlapped step (lbm.cu): after a bulk pass with
-// flags == nullptr, list the flagged segments (list: one int per segment at
-// most) and update their cells again with the force density and the
-// moments, 8-cell quarter by quarter: the quarters marked in `fine` (4 bytes
-// per segment, 4-byte aligned), all four of a flagged segment without
-// marks.  Flags and marks are cleared.  list: one int per quarter at most;
-// count: one int, reset here.  Three operations on stream s (a 4-byte
-// memset and two kernels).
+// Band cells of the overlapped step (lbm.cu).  launch_band_list lists the
+// flagged segments' 8-cell quarters: those marked in `fine` (4 bytes per
+// segment, 4-byte aligned), all four of a flagged segment without marks;
+// list: one int per quarter at most, *count has to be 0 and receives their
+// number, *next_count is set to 0.  launch_band_cells, after a bulk pass with
+// flags == nullptr, updates the listed cells again with the force density and
+// the moments and clears flags and marks.  One kernel each.
+void launch_band_list(const uint8_t* flags, const uint8_t* fine, const GridParams& g, int* list,
+                      int* count, int* next_count, cudaStream_t s);
 void launch_band_cells(int Q, int storage, const void* fin, void* fout, void* moments, void* F,
-                       uint8_t* flags, uint8_t* fine, int* list, int* count,
+                       uint8_t* flags, uint8_t* fine, const int* list, const int* count,
                        const StreamParams& p, int sm_count, cudaStream_t s);
 constexpr int BAND_KERNELS = 2;
 
@@ -340,7 +341,8 @@ __device__ __forceinline__ bool inside_cell(const int* __restrict__ cnt,
 }
 
 // Column crossings of the current interface (classify.cu); the column count
-// array is cleared first.
+// array has to be zero (launch_classify_clear).
+void launch_classify_clear(const GridParams& g, int* cnt, cudaStream_t s);
 void launch_classify(int dim, const double* q, int N, const int* tri, int M, const GridParams& g,
                      int* cnt, double* cz, int* err, cudaStream_t s);
 void launch_inside_mask(const GridParams& g, const int* cnt, const double* cz,

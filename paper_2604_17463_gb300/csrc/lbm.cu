@@ -348,13 +348,18 @@ static void launch_sc_t(bool write_all, const void* fin, void* fout, void* mom, 
 // band pass took the union, measured no faster: the plain kernel then has to
 // read the mark before its loads.)
 // One atomic per block of BAND_LIST_THREADS segments: the warps' counts
-// are summed in shared memory, thread 0 reserves the block's range.
+// are summed in shared memory, thread 0 reserves the block's range.  The list
+// needs the spread only, so it is made beside the bulk pass; it clears the
+// counter of the next step (two take turns) instead of a memset node, which
+// costs a step about 3 us.  With list and memset after the bulk pass the step
+// of the 256 x 256 x 128 drop (40 962 nodes) took 219 us, so 211.
 constexpr int BAND_LIST_THREADS = 256;
 
 __global__ void __launch_bounds__(BAND_LIST_THREADS)
 k_band_list(const uint8_t* __restrict__ flags, const uint8_t* __restrict__ fine, long long nseg,
-            int* __restrict__ list, int* __restrict__ count)
+            int* __restrict__ list, int* __restrict__ count, int* __restrict__ next_count)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *next_count = 0;  // the next step's counter
     __shared__ int s_cnt[BAND_LIST_THREADS / 32];
     __shared__ int s_base;
     // one thread per segment: its marked quarters (all four when flagged
@@ -427,30 +432,34 @@ k_band_sc(const typename StorageT<ST>::S* __restrict__ fin,
     }
 }
 
+void launch_band_list(const uint8_t* flags, const uint8_t* fine, const GridParams& g, int* list,
+                      int* count, int* next_count, cudaStream_t s)
+{
+    const long long nseg = (long long)g.ny * g.nz * g.nseg_x;
+    k_band_list<<<(unsigned)((nseg + BAND_LIST_THREADS - 1) / BAND_LIST_THREADS),
+                  BAND_LIST_THREADS, 0, s>>>(flags, fine, nseg, list, count, next_count);
+}
+
 template <int Q, int ST>
 static void launch_band_t(const void* fin, void* fout, void* mom, void* F, uint8_t* flags,
-                          uint8_t* fine, int* list, int* count, const StreamParams& p,
+                          uint8_t* fine, const int* list, const int* count, const StreamParams& p,
                           int sm_count, cudaStream_t s)
 {
     using T = StorageT<ST>;
-    const long long nseg = (long long)p.g.ny * p.g.nz * p.g.nseg_x;
-    cudaMemsetAsync(count, 0, sizeof(int), s);
-    k_band_list<<<(unsigned)((nseg + BAND_LIST_THREADS - 1) / BAND_LIST_THREADS),
-                  BAND_LIST_THREADS, 0, s>>>(flags, fine, nseg, list, count);
     auto* a = (const typename T::S*)fin;
     auto* b = (typename T::S*)fout;
     auto* m = (typename T::R*)mom;
     auto* f = (typename T::R*)F;
     // four listed quarters per warp, 16 blocks of 4 warps per SM
     const int grid = 16 * sm_count;
-    if (p.moving)
+    if (p.moving || p.two_tau)
         k_band_sc<Q, ST, true><<<grid, 128, 0, s>>>(a, b, m, f, flags, fine, list, count, p);
     else
         k_band_sc<Q, ST, false><<<grid, 128, 0, s>>>(a, b, m, f, flags, fine, list, count, p);
 }
 
 void launch_band_cells(int Q, int storage, const void* fin, void* fout, void* moments, void* F,
-                       uint8_t* flags, uint8_t* fine, int* list, int* count,
+                       uint8_t* flags, uint8_t* fine, const int* list, const int* count,
                        const StreamParams& p, int sm_count, cudaStream_t s)
 {
 #define IBLB_BAND(QQ, SS) \
