@@ -1058,7 +1058,7 @@ iblb_status iblb_batch_create(int lattice, int storage, size_t hbm_budget_bytes,
     if (e == cudaSuccess) e = cudaMalloc(&b->arena_ptr, budget);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_slots, sizeof(SlotDev) * max_slots);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_partial, sizeof(double) * 1024);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_obs, sizeof(double) * 12);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_obs, sizeof(double) * OBS_DOUBLES);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         iblb_batch_destroy(b);
@@ -1429,8 +1429,8 @@ iblb_status iblb_batch_observables(iblb_batch b, int slot, iblb_obs* out)
     launch_mass_partials(b->Q, b->storage, d.f[sl.buf], d.g, d.inv_scale, b->d_partial, b->stream);
     launch_observables(b->dim, d.q, d.N, b->dim == 3 ? d.tri : nullptr, d.M, b->d_partial,
                        mass_partial_blocks(d.g), sl.cfg.xi, 0.5, b->d_obs, b->stream);
-    b->launches += 2;
-    add_launches(2);
+    b->launches += 1 + OBS_KERNELS;
+    add_launches(1 + OBS_KERNELS);
     BCK(b, cudaGetLastError());
     double v[12];
     BCK(b, cudaMemcpyAsync(v, b->d_obs, sizeof(v), cudaMemcpyDeviceToHost, b->stream));

@@ -314,7 +314,11 @@ void launch_interp_grouped(int storage, double* q, const void* moments, const No
 void launch_elastic_reference(int dim, const double* q, int N, int M, const int* tri, double* eref,
                               cudaStream_t s);
 
-// Observables (single block, deterministic).  out: 12 doubles, layout of iblb_obs.
+// Observables (deterministic; OBS_KERNELS kernels).  out: OBS_DOUBLES doubles,
+// the first 12 the results in the layout of iblb_obs, the rest workspace.
+constexpr int OBS_GRID = 64;
+constexpr int OBS_DOUBLES = 16 + 30 * OBS_GRID;
+constexpr int OBS_KERNELS = 4;
 void launch_observables(int dim, const double* q, int N, const int* tri, int M,
                         const double* mass_partial, int n_partial, double xi, double wall_plane,
                         double* out, cudaStream_t s);

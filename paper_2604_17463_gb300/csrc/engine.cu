@@ -61,7 +61,7 @@ struct iblb_sim {
     int* err = nullptr;
     double* partial = nullptr;
     int npartial = 0;
-    double* obs = nullptr;     // 12 doubles
+    double* obs = nullptr;     // OBS_DOUBLES
     // interface
     int N = 0, M = 0;
     double* q = nullptr;         // node positions
@@ -574,7 +574,7 @@ iblb_status iblb_create(const iblb_config* cfg, void* cuda_stream, iblb_handle* 
     h->npartial = mass_partial_blocks(g);
     if ((e = cudaMalloc(&h->partial, sizeof(double) * h->npartial)) != cudaSuccess)
         return bail(e, "partial");
-    if ((e = cudaMalloc(&h->obs, sizeof(double) * 12)) != cudaSuccess) return bail(e, "obs");
+    if ((e = cudaMalloc(&h->obs, sizeof(double) * OBS_DOUBLES)) != cudaSuccess) return bail(e, "obs");
     if ((e = cudaMalloc(&h->defo, sizeof(double) * 8)) != cudaSuccess) return bail(e, "obs");
     if ((e = cudaMalloc(&h->rng, sizeof(unsigned) * 2)) != cudaSuccess) return bail(e, "obs");
     cudaMemsetAsync(h->rng, 0, sizeof(unsigned) * 2, h->stream);
@@ -912,7 +912,7 @@ iblb_status iblb_observables(iblb_handle h, iblb_obs* out)
                          h->stream);
     launch_observables(h->dim, h->q, h->N, h->tri, h->M, h->partial, h->npartial, h->cfg.xi, 0.5,
                        h->obs, h->stream);
-    g_launches += 2;
+    g_launches += 1 + OBS_KERNELS;
     CK(h, cudaGetLastError());
     double v[12];
     CK(h, cudaMemcpyAsync(v, h->obs, sizeof(v), cudaMemcpyDeviceToHost, h->stream));

@@ -219,15 +219,15 @@ void launch_interp(int storage, int dim, double* q, const void* moments, int N, 
 }
 
 // ------------------------------------------------------------------ A7 observables
-// Single block, fixed thread -> item assignment and reduction tree, so the
-// result is deterministic.  Contact-angle estimator: algebraic least-squares
-// circle (2D) / sphere (3D) through the nodes with d > 3 xi, centred on their
-// mean, intersected with the plane d = min_j d_j.
+// Fixed thread -> item assignment and reduction trees, so the results are
+// deterministic.  Contact-angle estimator: algebraic least-squares circle
+// (2D) / sphere (3D) through the nodes with d > 3 xi, centred on their mean,
+// intersected with the plane d = min_j d_j.
 constexpr int OBS_BLOCK = 1024;
-constexpr int OBS_MAXV = 20;
 
 // Reduce nv values per thread to thread 0 (sum), in a fixed order.
-__device__ void block_sum(double* v, int nv, double (*sh)[OBS_BLOCK / 32])
+template <int B>
+__device__ void block_sum(double* v, int nv, double (*sh)[B / 32])
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int k = 0; k < nv; k++) {
@@ -239,14 +239,15 @@ __device__ void block_sum(double* v, int nv, double (*sh)[OBS_BLOCK / 32])
     if (threadIdx.x == 0) {
         for (int k = 0; k < nv; k++) {
             double t = 0.0;
-            for (int w = 0; w < OBS_BLOCK / 32; w++) t += sh[k][w];
+            for (int w = 0; w < B / 32; w++) t += sh[k][w];
             v[k] = t;
         }
     }
     __syncthreads();
 }
 
-__device__ void block_minmax(double& mn, double& mx, double (*sh)[OBS_BLOCK / 32])
+template <int B>
+__device__ void block_minmax(double& mn, double& mx, double (*sh)[B / 32])
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int o = 16; o > 0; o >>= 1) {
@@ -259,7 +260,7 @@ __device__ void block_minmax(double& mn, double& mx, double (*sh)[OBS_BLOCK / 32
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 0; w < OBS_BLOCK / 32; w++) {
+        for (int w = 0; w < B / 32; w++) {
             mn = fmin(mn, sh[0][w]);
             mx = fmax(mx, sh[1][w]);
         }
@@ -298,84 +299,158 @@ __device__ bool solve_small(int n, double* A, double* b)
     return true;
 }
 
-__global__ void __launch_bounds__(OBS_BLOCK)
-k_observables(int dim, const double* __restrict__ q, int N, const int* __restrict__ tri, int M,
-              const double* __restrict__ mass_partial, int n_partial, double xi, double wp,
-              double* out)
+// The three passes of the observables (sums and extremes; normal equations of
+// the fit; film under the drop) and the last sum, one kernel each over up to
+// OBS_GRID blocks: a pass's blocks each add up the previous pass's partial
+// sums for themselves.  FP64 arithmetic bounds them: in one block, on one SM's
+// pipe, the call (with the mass sum and its synchronisations) took 0.16 ms on
+// the 128 x 64 ring, 0.41 ms with 10 242 nodes and 1.63 ms with 40 962; so 0.12,
+// 0.16 and 0.79 ms.
+constexpr int OBS_THREADS = 256;
+constexpr int OBS_P1 = 8, OBS_P2 = 20, OBS_P3 = 2;  // doubles per block and pass
+
+struct ObsArgs {
+    int dim;
+    const double* q;
+    int N;
+    const int* tri;
+    int M;
+    const double* mass_partial;
+    int n_partial;
+    double xi, wp;
+    double* out;           // 12 results
+    double *p1, *p2, *p3;  // partial sums [OBS_GRID][...]
+};
+
+// Sums over the blocks of column k of a partial array, by the first warp
+// (ascending rows per lane, then a fixed tree).
+__device__ __forceinline__ double column_sum(const double* p, int stride, int k, int grid)
 {
-    __shared__ double sh[OBS_MAXV][OBS_BLOCK / 32];
-    __shared__ double bc[8];
-    const int t = threadIdx.x;
-    const int wax = dim - 1;
-    // phase 1: mass, volume, extremes, mean of the fit set
-    double v[OBS_MAXV];
-    for (int k = 0; k < OBS_MAXV; k++) v[k] = 0.0;
-    for (int b = t; b < n_partial; b += OBS_BLOCK) v[0] += mass_partial[b];
+    double s = 0.0;
+    for (int r = threadIdx.x; r < grid; r += 32) s += p[r * stride + k];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+__global__ void __launch_bounds__(OBS_THREADS) k_obs_sums(ObsArgs a)
+{
+    __shared__ double sh[6][OBS_THREADS / 32];
+    const int t0 = blockIdx.x * OBS_THREADS + threadIdx.x, nt = gridDim.x * OBS_THREADS;
+    const int dim = a.dim, wax = dim - 1;
+    const double* q = a.q;
+    double v[6] = {0, 0, 0, 0, 0, 0};  // mass, volume, sum of the fit set (3), its count
+    for (int b = t0; b < a.n_partial; b += nt) v[0] += a.mass_partial[b];
     if (dim == 2) {
-        for (int j = t; j < N; j += OBS_BLOCK) {
-            const int jn = (j + 1 == N) ? 0 : j + 1;
+        for (int j = t0; j < a.N; j += nt) {
+            const int jn = (j + 1 == a.N) ? 0 : j + 1;
             v[1] += q[2 * j] * q[2 * jn + 1] - q[2 * jn] * q[2 * j + 1];
         }
     } else {
-        for (int f = t; f < M; f += OBS_BLOCK) {
-            const double* a = q + 3 * tri[3 * f];
-            const double* b = q + 3 * tri[3 * f + 1];
-            const double* c = q + 3 * tri[3 * f + 2];
-            v[1] += a[0] * (b[1] * c[2] - b[2] * c[1]) + a[1] * (b[2] * c[0] - b[0] * c[2]) +
-                    a[2] * (b[0] * c[1] - b[1] * c[0]);
+        for (int f = t0; f < a.M; f += nt) {
+            const double* x = q + 3 * a.tri[3 * f];
+            const double* y = q + 3 * a.tri[3 * f + 1];
+            const double* z = q + 3 * a.tri[3 * f + 2];
+            v[1] += x[0] * (y[1] * z[2] - y[2] * z[1]) + x[1] * (y[2] * z[0] - y[0] * z[2]) +
+                    x[2] * (y[0] * z[1] - y[1] * z[0]);
         }
     }
     double hmin = 1e300, hmax = -1e300;
-    for (int j = t; j < N; j += OBS_BLOCK) {
+    for (int j = t0; j < a.N; j += nt) {
         const double h = q[dim * j + wax];
         hmin = fmin(hmin, h);
         hmax = fmax(hmax, h);
-        if (h - wp > 3.0 * xi) {
+        if (h - a.wp > 3.0 * a.xi) {
             for (int k = 0; k < dim; k++) v[2 + k] += q[dim * j + k];
             v[5] += 1.0;
         }
     }
-    block_sum(v, 6, sh);
-    block_minmax(hmin, hmax, sh);
-    if (t == 0) {
-        out[0] = v[0];
-        out[1] = (dim == 2) ? 0.5 * v[1] : v[1] / 6.0;
-        out[2] = hmax - hmin;
-        out[6] = hmin - wp;
-        bc[0] = v[5];
-        for (int k = 0; k < dim; k++) bc[1 + k] = v[5] > 0 ? v[2 + k] / v[5] : 0.0;
+    block_sum<OBS_THREADS>(v, 6, sh);
+    block_minmax<OBS_THREADS>(hmin, hmax, sh);
+    if (threadIdx.x == 0) {
+        double* r = a.p1 + OBS_P1 * blockIdx.x;
+        for (int k = 0; k < 6; k++) r[k] = v[k];
+        r[6] = hmin;
+        r[7] = hmax;
     }
+}
+
+__global__ void __launch_bounds__(OBS_THREADS) k_obs_fit(ObsArgs a)
+{
+    __shared__ double sh[OBS_P2][OBS_THREADS / 32];
+    __shared__ double tot[6];
+    const int dim = a.dim, wax = dim - 1, np = dim + 1;
+    if (threadIdx.x < 32)
+        for (int k = 0; k < 6; k++) {
+            const double s = column_sum(a.p1, OBS_P1, k, gridDim.x);
+            if (threadIdx.x == 0) tot[k] = s;
+        }
     __syncthreads();
-    const double cnt = bc[0];
-    const double mean[3] = {bc[1], bc[2], dim == 3 ? bc[3] : 0.0};
-    __syncthreads();
-    // phase 2: normal equations of the algebraic fit
-    const int np = dim + 1;
-    for (int k = 0; k < OBS_MAXV; k++) v[k] = 0.0;
-    for (int j = t; j < N; j += OBS_BLOCK) {
-        if (!(q[dim * j + wax] - wp > 3.0 * xi)) continue;
+    const double cnt = tot[5];
+    double mean[3] = {0, 0, 0};
+    for (int k = 0; k < dim; k++) mean[k] = cnt > 0 ? tot[2 + k] / cnt : 0.0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        double hmin = 1e300, hmax = -1e300;
+        for (int r = 0; r < (int)gridDim.x; r++) {
+            hmin = fmin(hmin, a.p1[OBS_P1 * r + 6]);
+            hmax = fmax(hmax, a.p1[OBS_P1 * r + 7]);
+        }
+        a.out[0] = tot[0];
+        a.out[1] = (dim == 2) ? 0.5 * tot[1] : tot[1] / 6.0;
+        a.out[2] = hmax - hmin;
+        a.out[6] = hmin - a.wp;
+    }
+    double v[OBS_P2];
+    for (int k = 0; k < OBS_P2; k++) v[k] = 0.0;
+    const double* q = a.q;
+    for (int j = blockIdx.x * OBS_THREADS + threadIdx.x; j < a.N; j += gridDim.x * OBS_THREADS) {
+        if (!(q[dim * j + wax] - a.wp > 3.0 * a.xi)) continue;
         double vv[4], r2 = 0.0;
         for (int k = 0; k < dim; k++) {
             vv[k] = q[dim * j + k] - mean[k];
             r2 += vv[k] * vv[k];
         }
         vv[dim] = 1.0;
-        for (int a = 0; a < np; a++) {
-            for (int b = 0; b < np; b++) v[a * np + b] += vv[a] * vv[b];
-            v[16 + a] -= vv[a] * r2;
+        for (int x = 0; x < np; x++) {
+            for (int y = 0; y < np; y++) v[x * np + y] += vv[x] * vv[y];
+            v[16 + x] -= vv[x] * r2;
         }
     }
-    block_sum(v, OBS_MAXV, sh);
-    if (t == 0) {
+    block_sum<OBS_THREADS>(v, OBS_P2, sh);
+    if (threadIdx.x == 0)
+        for (int k = 0; k < OBS_P2; k++) a.p2[OBS_P2 * blockIdx.x + k] = v[k];
+}
+
+__global__ void __launch_bounds__(OBS_THREADS) k_obs_film(ObsArgs a)
+{
+    __shared__ double sh[OBS_P3][OBS_THREADS / 32];
+    __shared__ double sums[OBS_P2], tot[6], bc[3];
+    const int dim = a.dim, np = dim + 1;
+    if (threadIdx.x < 32) {
+        for (int k = 2; k < 6; k++) {
+            const double s = column_sum(a.p1, OBS_P1, k, gridDim.x);
+            if (threadIdx.x == 0) tot[k] = s;
+        }
+        for (int k = 0; k < OBS_P2; k++) {
+            const double s = column_sum(a.p2, OBS_P2, k, gridDim.x);
+            if (threadIdx.x == 0) sums[k] = s;
+        }
+    }
+    __syncthreads();
+    double* out = a.out;
+    const bool writer = blockIdx.x == 0;
+    if (threadIdx.x == 0) {
+        const double cnt = tot[5];
         bool ok = cnt >= dim + 1;
         double Am[16], rhs[4];
-        for (int k = 0; k < np * np; k++) Am[k] = v[k];
-        for (int k = 0; k < np; k++) rhs[k] = v[16 + k];
+        for (int k = 0; k < np * np; k++) Am[k] = sums[k];
+        for (int k = 0; k < np; k++) rhs[k] = sums[16 + k];
         if (ok) ok = solve_small(np, Am, rhs);
         if (!ok) {
-            out[3] = out[4] = out[5] = out[11] = nan("");
-            out[7] = out[8] = out[9] = 0.0;
-            bc[4] = -1.0;
+            if (writer) {
+                out[3] = out[4] = out[5] = out[11] = nan("");
+                out[7] = out[8] = out[9] = 0.0;
+            }
+            bc[0] = -1.0;
         } else {
             double cen[3] = {0, 0, 0}, R2 = 0.0;
             for (int k = 0; k < dim; k++) {
@@ -384,32 +459,33 @@ k_observables(int dim, const double* __restrict__ q, int N, const int* __restric
             }
             R2 -= rhs[dim];
             const double R = sqrt(R2);
-            for (int k = 0; k < dim; k++) cen[k] += mean[k];
-            const double plane = wp + out[6];
-            const double dz = plane - cen[dim - 1];
-            double cth = dz / R;
-            cth = fmin(1.0, fmax(-1.0, cth));
-            out[3] = acos(cth) * (180.0 / 3.141592653589793);
+            for (int k = 0; k < dim; k++) cen[k] += cnt > 0 ? tot[2 + k] / cnt : 0.0;
+            double hmin = 1e300;
+            for (int r = 0; r < (int)gridDim.x; r++) hmin = fmin(hmin, a.p1[OBS_P1 * r + 6]);
+            const double dz = a.wp + (hmin - a.wp) - cen[dim - 1];
             const double rc2 = R * R - dz * dz;
-            out[4] = rc2 > 0.0 ? sqrt(rc2) : 0.0;
-            out[7] = cen[0];
-            out[8] = cen[1];
-            out[9] = cen[2];
-            out[10] = R;
-            bc[4] = out[4];
-            bc[5] = cen[0];
-            bc[6] = cen[1];
+            const double rc = rc2 > 0.0 ? sqrt(rc2) : 0.0;
+            if (writer) {
+                const double cth = fmin(1.0, fmax(-1.0, dz / R));
+                out[3] = acos(cth) * (180.0 / 3.141592653589793);
+                out[4] = rc;
+                out[7] = cen[0];
+                out[8] = cen[1];
+                out[9] = cen[2];
+                out[10] = R;
+            }
+            bc[0] = rc;
+            bc[1] = cen[0];
+            bc[2] = cen[1];
         }
     }
     __syncthreads();
-    const double rcl = bc[4];
-    const double c0 = bc[5], c1 = bc[6];
-    __syncthreads();
-    // phase 3: film thickness under the drop
-    for (int k = 0; k < OBS_MAXV; k++) v[k] = 0.0;
+    const double rcl = bc[0], c0 = bc[1], c1 = bc[2];
+    double v[OBS_P3] = {0, 0};
     if (rcl >= 0.0) {
-        for (int j = t; j < N; j += OBS_BLOCK) {
-            const double d = q[dim * j + wax] - wp;
+        const double* q = a.q;
+        for (int j = blockIdx.x * OBS_THREADS + threadIdx.x; j < a.N; j += gridDim.x * OBS_THREADS) {
+            const double d = q[dim * j + dim - 1] - a.wp;
             double rr = 0.0;
             const double t0 = q[dim * j] - c0;
             rr += t0 * t0;
@@ -417,19 +493,26 @@ k_observables(int dim, const double* __restrict__ q, int N, const int* __restric
                 const double t1 = q[dim * j + 1] - c1;
                 rr += t1 * t1;
             }
-            if (sqrt(rr) < 0.5 * rcl && d <= 3.0 * xi) {
+            if (sqrt(rr) < 0.5 * rcl && d <= 3.0 * a.xi) {
                 v[0] += d;
                 v[1] += 1.0;
             }
         }
     }
-    block_sum(v, 2, sh);
-    if (t == 0) {
-        if (rcl >= 0.0) out[5] = v[1] > 0 ? v[0] / v[1] : nan("");
-        if (N == 0) {
-            for (int k = 1; k < 12; k++) out[k] = 0.0;
-        }
+    block_sum<OBS_THREADS>(v, OBS_P3, sh);
+    if (threadIdx.x == 0) {
+        a.p3[OBS_P3 * blockIdx.x] = v[0];
+        a.p3[OBS_P3 * blockIdx.x + 1] = rcl >= 0.0 ? v[1] : -1.0;  // no fit: no film
     }
+}
+
+__global__ void __launch_bounds__(32) k_obs_last(ObsArgs a, int grid)
+{
+    const double d = column_sum(a.p3, OBS_P3, 0, grid), n = column_sum(a.p3, OBS_P3, 1, grid);
+    if (threadIdx.x != 0) return;
+    if (n >= 0.0) a.out[5] = n > 0 ? d / n : nan("");
+    if (a.N == 0)
+        for (int k = 1; k < 12; k++) a.out[k] = 0.0;
 }
 
 // Deformation index (Sec. 4, Eq. 15): the enclosed region is split into
@@ -451,7 +534,7 @@ k_deformation(int dim, const double* __restrict__ q, int N, const int* __restric
     for (int k = 0; k < 6; k++) v[k] = 0.0;
     for (int j = t; j < N; j += OBS_BLOCK)
         for (int k = 0; k < dim; k++) v[k] += q[dim * j + k];
-    block_sum(v, 3, sh);
+    block_sum<OBS_BLOCK>(v, 3, sh);
     if (t == 0)
         for (int k = 0; k < 3; k++) p0s[k] = k < dim ? v[k] / N : 0.0;
     __syncthreads();
@@ -489,7 +572,7 @@ k_deformation(int dim, const double* __restrict__ q, int N, const int* __restric
         v[4] += f2 * (a[w] * a[w] + b[w] * b[w] + c[w] * c[w] + sw * sw);
         v[5] += f2 * (a[0] * a[w] + b[0] * b[w] + c[0] * c[w] + sx * sw);
     }
-    block_sum(v, 6, sh);
+    block_sum<OBS_BLOCK>(v, 6, sh);
     if (t == 0) {
         const double vol = v[0];
         const double gx = v[1] / vol, gw = v[2] / vol;
@@ -518,8 +601,17 @@ void launch_observables(int dim, const double* q, int N, const int* tri, int M,
                         const double* mass_partial, int n_partial, double xi, double wall_plane,
                         double* out, cudaStream_t s)
 {
-    k_observables<<<1, OBS_BLOCK, 0, s>>>(dim, q, N, tri, M, mass_partial, n_partial, xi,
-                                          wall_plane, out);
+    ObsArgs a{dim, q, N, tri, M, mass_partial, n_partial, xi, wall_plane, out, nullptr, nullptr, nullptr};
+    a.p1 = out + 16;
+    a.p2 = a.p1 + OBS_P1 * OBS_GRID;
+    a.p3 = a.p2 + OBS_P2 * OBS_GRID;
+    static_assert(16 + (OBS_P1 + OBS_P2 + OBS_P3) * OBS_GRID <= OBS_DOUBLES, "observables workspace");
+    int grid = ((N > n_partial ? N : n_partial) + OBS_THREADS - 1) / OBS_THREADS;
+    grid = grid < 1 ? 1 : (grid > OBS_GRID ? OBS_GRID : grid);
+    k_obs_sums<<<grid, OBS_THREADS, 0, s>>>(a);
+    k_obs_fit<<<grid, OBS_THREADS, 0, s>>>(a);
+    k_obs_film<<<grid, OBS_THREADS, 0, s>>>(a);
+    k_obs_last<<<1, 32, 0, s>>>(a, grid);
 }
 
 }  // namespace iblb
