@@ -44,6 +44,7 @@ struct SlotDev {
     unsigned* rng;         // two-entry step counter for binary16 stochastic rounding
     int cpt;               // 32-cell row segments per stream-collide work item
     double* q;
+    double* q2;                 // second position buffer of the fused ring kernel (2D)
     double* phi;
     int N, M;
     int* tri;
@@ -391,18 +392,48 @@ k_b_spread(const SlotDev* __restrict__ slots, const int2* __restrict__ nodes, in
     spread_node<D, R>(sd.g, sd.q, sd.phi, nd.y, (R*)sd.F, sd.flags);
 }
 
-// One thread per (slot, node): interpolate and advect (interp_node).
+// One thread per (slot, node): interpolate and advect (interp_node).  The
+// positions are read from the second buffer when `sel` is set, and written to
+// the first.
 template <int D, typename R>
 __global__ void __launch_bounds__(128)
-k_b_interp(const SlotDev* __restrict__ slots, const int2* __restrict__ nodes, int nnodes)
+k_b_interp(const SlotDev* __restrict__ slots, const int2* __restrict__ nodes, int nnodes, int sel)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nnodes) return;
     const int2 nd = nodes[t];
     const SlotDev& sd = slots[nd.x];
+    const double* q = (D == 2 && sel) ? sd.q2 : sd.q;
     R acc[3];
-    interp_node<D, R>(sd.g, sd.q, (const R*)sd.mom, nd.y, acc);
-    for (int k = 0; k < D; k++) sd.q[D * nd.y + k] += (double)acc[k];
+    interp_node<D, R>(sd.g, q, (const R*)sd.mom, nd.y, acc);
+    for (int k = 0; k < D; k++) sd.q[D * nd.y + k] = q[D * nd.y + k] + (double)acc[k];
+}
+
+// Rings between two stream-collides, one warp per (slot, first node) item
+// (ring_warp): advection with the last step's velocity, forces, spread; from
+// the buffer `sel` into the other.
+template <typename R, bool FIRST>
+__global__ void __launch_bounds__(32)
+k_b_ring(const SlotDev* __restrict__ slots, const int2* __restrict__ rings, int sel)
+{
+    const int2 it = rings[blockIdx.x];
+    const SlotDev& sd = slots[it.x];
+    ring_warp<R, FIRST>(sd.g, sel ? sd.q2 : sd.q, sel ? sd.q : sd.q2, sd.N, it.y, sd.fp,
+                        (const R*)sd.mom, (R*)sd.F, sd.flags, sd.err);
+}
+
+// One thread per (slot, node) of the meshes: force from the face records, then
+// its spread.
+template <typename R>
+__global__ void __launch_bounds__(64)
+k_b_node_spread(const SlotDev* __restrict__ slots, const int2* __restrict__ nodes, int nnodes)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nnodes) return;
+    const int2 nd = nodes[t];
+    const SlotDev& sd = slots[nd.x];
+    mesh_node_spread<R>(sd.g, sd.q, nd.y, sd.entry_rec, sd.csr_ptr, sd.fp, (R*)sd.F, sd.flags, nullptr,
+                        sd.err);
 }
 
 }  // namespace
@@ -472,7 +503,7 @@ __global__ void k_b_col_clear(const SlotDev* __restrict__ slots, const int* __re
 }
 
 __global__ void k_b_classify(const SlotDev* __restrict__ slots, const int2* __restrict__ items,
-                             int n, int dim)
+                             int n, int dim, int sel)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
@@ -480,13 +511,13 @@ __global__ void k_b_classify(const SlotDev* __restrict__ slots, const int2* __re
     const SlotDev& sd = slots[it.x];
     if (!sd.two_tau) return;
     if (dim == 2)
-        classify_segment(sd.q, sd.N, it.y, sd.g, sd.col_cnt, sd.col_z, sd.err);
+        classify_segment(sel ? sd.q2 : sd.q, sd.N, it.y, sd.g, sd.col_cnt, sd.col_z, sd.err);
     else
         classify_face(sd.q, sd.tri, it.y, sd.g, sd.col_cnt, sd.col_z, sd.err);
 }
 
 static void launch_b_ib(int dim, int storage, int phase, const SlotDev* slots, const int2* nodes,
-                        int nnodes, const int2* faces, int nfaces, cudaStream_t s)
+                        int nnodes, const int2* faces, int nfaces, cudaStream_t s, int sel = 0)
 {
     const int wb = 128;
     const int node_grid = (nnodes + wb - 1) / wb;  // one thread per (slot, node)
@@ -509,11 +540,11 @@ static void launch_b_ib(int dim, int storage, int phase, const SlotDev* slots, c
         }
     } else {  // interpolate + advect
         if (storage == ST_FP64) {
-            if (dim == 2) k_b_interp<2, double><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes);
-            else k_b_interp<3, double><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes);
+            if (dim == 2) k_b_interp<2, double><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes, sel);
+            else k_b_interp<3, double><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes, sel);
         } else {
-            if (dim == 2) k_b_interp<2, float><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes);
-            else k_b_interp<3, float><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes);
+            if (dim == 2) k_b_interp<2, float><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes, sel);
+            else k_b_interp<3, float><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes, sel);
         }
     }
 }
@@ -578,7 +609,7 @@ struct Arena {
 };
 
 struct Layout {
-    size_t pop[2], mom, F, flags, err, rng, q, phi, tri, csr, epos, erec, eref, cols, colz, total;
+    size_t pop[2], mom, F, flags, err, rng, q, q2, phi, tri, csr, epos, erec, eref, cols, colz, total;
 };
 
 Layout slot_layout(int Q, int dim, size_t elt, size_t relt, long long ncell, int rowlen, int N,
@@ -600,6 +631,7 @@ Layout slot_layout(int Q, int dim, size_t elt, size_t relt, long long ncell, int
     L.err = take(sizeof(int));
     L.rng = take(2 * sizeof(unsigned));
     L.q = take(sizeof(double) * (size_t)N * dim);
+    if (dim == 2 && elt != 2) L.q2 = take(sizeof(double) * (size_t)N * dim);
     L.phi = take(sizeof(double) * (size_t)N * dim);
     if (dim == 3) {
         L.tri = take(sizeof(int) * 3 * (size_t)M);
@@ -636,10 +668,26 @@ double wetting_A(const iblb_config& c)
 
 }  // namespace
 
+// A part of the active slots: ranges of the work lists (which are in slot
+// order).  A batch of meshes steps in two parts of about the same work on two
+// streams, so that one part's IB kernels, bound by latency, run beside the
+// other's stream-collide, bound by memory.
+struct Part {
+    int t0 = 0, t1 = 0;  // stream-collide items
+    int n0 = 0, n1 = 0;  // nodes
+    int f0 = 0, f1 = 0;  // faces
+    int r0 = 0, r1 = 0;  // warp pieces of rings
+    int c0 = 0, c1 = 0;  // slots with a viscosity ratio
+};
+
 struct iblb_batch_s {
     int Q = 9, dim = 2, storage = 0;
     size_t elt = 8, relt = 8;
-    cudaStream_t stream = nullptr, cap = nullptr;
+    cudaStream_t stream = nullptr;
+    // capture streams: the IB chain of each part at the highest priority, its
+    // stream-collides at the lowest
+    cudaStream_t cap[2] = {nullptr, nullptr}, low[2] = {nullptr, nullptr};
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_ib = nullptr, ev_sc = nullptr;
     unsigned char* arena_ptr = nullptr;
     Arena arena;
     std::vector<Slot> slots;
@@ -647,7 +695,9 @@ struct iblb_batch_s {
     BItem* d_tiles = nullptr;  // stream-collide work items
     int2* d_nodes = nullptr;
     int2* d_faces = nullptr;
-    size_t cap_tiles = 0, cap_nodes = 0, cap_faces = 0;
+    int2* d_rings = nullptr;
+    size_t cap_tiles = 0, cap_nodes = 0, cap_faces = 0, cap_rings = 0;
+    std::vector<Part> parts;
     int* d_tt = nullptr;      // active slots with a viscosity ratio
     size_t cap_tt = 0;
     int ntt = 0, max_ncol = 0;
@@ -741,12 +791,34 @@ void slot_items(const SlotDev& d, int slot, int cpt, std::vector<BItem>& out)
         }
 }
 
+// Whether the active slots step in two parts: meshes only, at least two slots
+// with enough cells that a part's stream-collide is worth hiding something
+// behind (2^18: about 5 us).  8 requests of 64^3 to 192 x 192 x 96 in FP32:
+// 441 us per step in two parts, 516 in one.  Rings gain nothing (their IB
+// kernel is shorter than what the second chain of launches costs: 48 FP32
+// drops 75 against 70 ms, 64 binary16 drops 46.6 against 46.5 us per step).
+// The ordered spread bins all slots together.
+bool two_parts(const iblb_batch_s* b, long long cells)
+{
+    return b->dim == 3 && !b->det && b->nactive >= 2 && cells >= (1LL << 18);
+}
+
+// The fused IB kernels: rings in FP64 and FP32, meshes; not with the ordered
+// spread.
+bool ring_fused(const iblb_batch_s* b) { return b->dim == 2 && b->storage != IBLB_FP16_DEV && !b->det; }
+bool mesh_fused(const iblb_batch_s* b) { return b->dim == 3 && !b->det; }
+
 // Rebuild the slot descriptors and the work lists of the active slots.
 iblb_status rebuild(iblb_batch_s* b)
 {
     std::vector<BItem> tiles;
-    std::vector<int2> nodes, faces;
+    std::vector<int2> nodes, faces, rings;
     std::vector<SlotDev> devs(b->slots.size());
+    // cells of the active slots, and the list positions where each begins
+    std::vector<long long> cells_before;
+    std::vector<Part> begins;
+    long long cells = 0;
+    int n_tt = 0;
     for (size_t s = 0; s < b->slots.size(); s++) {
         Slot& sl = b->slots[s];
         if (!sl.used) continue;
@@ -754,6 +826,18 @@ iblb_status rebuild(iblb_batch_s* b)
         sl.dev.cpt = sl.cpt;
         devs[s] = sl.dev;
         if (!sl.active) continue;
+        Part at;
+        at.t0 = (int)tiles.size();
+        at.n0 = (int)nodes.size();
+        at.f0 = (int)faces.size();
+        at.r0 = (int)rings.size();
+        at.c0 = n_tt;
+        begins.push_back(at);
+        cells_before.push_back(cells);
+        cells += sl.dev.nfluid;
+        n_tt += sl.dev.two_tau;
+        if (b->dim == 2)
+            for (int j = 0; j < sl.dev.N; j += RING_OWN) rings.push_back(make_int2((int)s, j));
         slot_items(sl.dev, (int)s, sl.cpt, tiles);
         for (int j = 0; j < sl.dev.N; j++) nodes.push_back(make_int2((int)s, j));
         for (int f = 0; f < (b->dim == 3 ? sl.dev.M : 0); f++) faces.push_back(make_int2((int)s, f));
@@ -762,6 +846,9 @@ iblb_status rebuild(iblb_batch_s* b)
     BCK(b, ensure(&b->d_tiles, &b->cap_tiles, tiles.size()));
     BCK(b, ensure(&b->d_nodes, &b->cap_nodes, nodes.size()));
     BCK(b, ensure(&b->d_faces, &b->cap_faces, faces.size()));
+    BCK(b, ensure(&b->d_rings, &b->cap_rings, rings.size()));
+    if (!rings.empty())
+        BCK(b, cudaMemcpy(b->d_rings, rings.data(), sizeof(int2) * rings.size(), cudaMemcpyHostToDevice));
     if (!devs.empty())
         BCK(b, cudaMemcpy(b->d_slots, devs.data(), sizeof(SlotDev) * devs.size(),
                           cudaMemcpyHostToDevice));
@@ -836,6 +923,25 @@ iblb_status rebuild(iblb_batch_s* b)
     int na = 0;
     for (auto& sl : b->slots) na += sl.active ? 1 : 0;
     b->nactive = na;
+    Part all;
+    all.t1 = b->ntiles;
+    all.n1 = b->nnodes;
+    all.f1 = b->nfaces;
+    all.r1 = (int)rings.size();
+    all.c1 = b->ntt;
+    b->parts.assign(1, all);
+    if (two_parts(b, cells)) {
+        size_t cut = 1;  // the slot boundary nearest to half the cells
+        for (size_t k = 1; k < begins.size(); k++)
+            if (std::llabs(2 * cells_before[k] - cells) < std::llabs(2 * cells_before[cut] - cells)) cut = k;
+        Part lo = all, hi = all;
+        lo.t1 = hi.t0 = begins[cut].t0;
+        lo.n1 = hi.n0 = begins[cut].n0;
+        lo.f1 = hi.f0 = begins[cut].f0;
+        lo.r1 = hi.r0 = begins[cut].r0;
+        lo.c1 = hi.c0 = begins[cut].c0;
+        b->parts = {lo, hi};
+    }
     clear_graphs(b);
     b->dirty = false;
     return IBLB_OK;
@@ -847,43 +953,106 @@ int kernels_per_step(const iblb_batch_s* b)
     return (b->dim == 3 ? 2 : 1) + 2 + (b->det ? DET_KERNELS : 1) + (b->ntt > 0 ? 2 : 0);
 }
 
-// Viscosity ratio: inside / outside of every slot that has one, from the
-// interface at the start of the step (before its stream-collide).
-void enqueue_classify(iblb_batch_s* b, cudaStream_t s)
+// Kernels of a replayed chunk of k steps.
+long long graph_kernels(const iblb_batch_s* b, int k)
 {
-    if (b->ntt == 0 || b->nnodes == 0) return;
-    k_b_col_clear<<<dim3((b->max_ncol + 255) / 256, b->ntt), 256, 0, s>>>(b->d_slots, b->d_tt);
-    const int2* items = b->dim == 2 ? b->d_nodes : b->d_faces;
-    const int n = b->dim == 2 ? b->nnodes : b->nfaces;
-    k_b_classify<<<(n + 127) / 128, 128, 0, s>>>(b->d_slots, items, n, b->dim);
+    long long n = 0;
+    for (const Part& p : b->parts) {
+        const int cl = p.c1 > p.c0 ? 2 : 0;
+        if (p.n1 == p.n0) n += k;
+        else if (ring_fused(b)) n += (long long)k * (2 + cl) + 1;
+        else if (mesh_fused(b)) n += (long long)k * (4 + cl);
+        else n += (long long)k * kernels_per_step(b);
+    }
+    return n;
 }
 
-// A2/A3 over all active slots: atomics, or the ordered gather.
-void enqueue_spread(iblb_batch_s* b, cudaStream_t s)
+// Viscosity ratio: inside / outside of every slot of a part that has one, from
+// the interface at the start of the step (before its stream-collide), in the
+// position buffer `sel`.
+void enqueue_classify(iblb_batch_s* b, cudaStream_t s, const Part& p, int sel = 0)
 {
-    if (b->det)
+    if (p.c1 == p.c0 || p.n1 == p.n0) return;
+    k_b_col_clear<<<dim3((b->max_ncol + 255) / 256, p.c1 - p.c0), 256, 0, s>>>(b->d_slots, b->d_tt + p.c0);
+    const int2* items = b->dim == 2 ? b->d_nodes + p.n0 : b->d_faces + p.f0;
+    const int n = b->dim == 2 ? p.n1 - p.n0 : p.f1 - p.f0;
+    k_b_classify<<<(n + 127) / 128, 128, 0, s>>>(b->d_slots, items, n, b->dim, sel);
+}
+
+// A2/A3 over a part's slots: atomics, or the ordered gather (all slots).
+void enqueue_spread(iblb_batch_s* b, cudaStream_t s, const Part& p)
+{
+    if (b->det) {
         launch_spread_det(b->storage, b->dim, b->d_detslots, b->d_nodes, b->nnodes, b->detb,
                           b->det_nbins, b->det_ncelltiles, b->sm_count, s);
-    else
-        launch_b_ib(b->dim, b->storage, 1, b->d_slots, b->d_nodes, b->nnodes, b->d_faces,
-                    b->nfaces, s);
+        return;
+    }
+    launch_b_ib(b->dim, b->storage, 1, b->d_slots, b->d_nodes + p.n0, p.n1 - p.n0, nullptr, 0, s);
 }
 
-// One batched step at parity `par` (all phases over all active slots).
-void enqueue_step(iblb_batch_s* b, cudaStream_t s, int par, bool write_all)
+// With two parts the blocks are short-lived (SC_ITEMS items per warp) instead
+// of persistent, so that the other part's IB kernels find room on the SMs: a
+// persistent launch holds all registers until it ends (the 8 requests above:
+// 492 us persistent, 514, 485, 442 and 441 with 16, 8, 4 and 2 items).
+constexpr int SC_ITEMS = 2;
+
+void enqueue_sc(iblb_batch_s* b, cudaStream_t s, const Part& p, int par, bool write_all)
 {
-    if (b->nnodes > 0) {
-        launch_b_ib(b->dim, b->storage, 0, b->d_slots, b->d_nodes, b->nnodes, b->d_faces,
-                    b->nfaces, s);
-        enqueue_spread(b, s);
-        enqueue_classify(b, s);
+    const int n = p.t1 - p.t0;
+    const int most = b->parts.size() > 1 ? (n + SC_ITEMS * (BT / 32) - 1) / (SC_ITEMS * (BT / 32))
+                                         : b->sm_count * b->sc_blocks_per_sm;
+    const int grid = std::max(1, std::min(n, most));
+    launch_b_sc(b->Q, b->storage, write_all, b->any_ext, b->d_slots, b->d_tiles + p.t0, n, par, grid, s);
+}
+
+void enqueue_interp(iblb_batch_s* b, cudaStream_t s, const Part& p, int sel = 0)
+{
+    launch_b_ib(b->dim, b->storage, 2, b->d_slots, b->d_nodes + p.n0, p.n1 - p.n0, nullptr, 0, s, sel);
+}
+
+// `steps` batched steps of one part from parity `par`, all phases over its
+// slots; the stream-collides on stream `low`.  Fused rings end with their
+// positions in the first buffer.
+void enqueue_steps(iblb_batch_s* b, cudaStream_t s, cudaStream_t low, const Part& p, int par, int steps,
+                   bool last)
+{
+    const bool ib = p.n1 > p.n0, ring = ring_fused(b);
+    const int nr = p.r1 - p.r0, nn = p.n1 - p.n0, nf = p.f1 - p.f0;
+    int sel = 0;
+    for (int k = 0; k < steps; k++) {
+        const bool wa = last && k == steps - 1;
+        if (ib && ring) {
+            const int2* r = b->d_rings + p.r0;
+            if (b->storage == ST_FP64) {
+                if (k == 0) k_b_ring<double, true><<<nr, 32, 0, s>>>(b->d_slots, r, sel);
+                else k_b_ring<double, false><<<nr, 32, 0, s>>>(b->d_slots, r, sel);
+            } else {
+                if (k == 0) k_b_ring<float, true><<<nr, 32, 0, s>>>(b->d_slots, r, sel);
+                else k_b_ring<float, false><<<nr, 32, 0, s>>>(b->d_slots, r, sel);
+            }
+            if (k > 0) sel ^= 1;
+        } else if (ib && mesh_fused(b)) {
+            k_b_face_geometry<<<(nf + 63) / 64, 64, 0, s>>>(b->d_slots, b->d_faces + p.f0, nf);
+            const int2* nd = b->d_nodes + p.n0;
+            if (b->storage == ST_FP64) k_b_node_spread<double><<<(nn + 63) / 64, 64, 0, s>>>(b->d_slots, nd, nn);
+            else k_b_node_spread<float><<<(nn + 63) / 64, 64, 0, s>>>(b->d_slots, nd, nn);
+        } else if (ib) {
+            launch_b_ib(b->dim, b->storage, 0, b->d_slots, b->d_nodes + p.n0, nn, b->d_faces + p.f0, nf, s);
+            enqueue_spread(b, s, p);
+        }
+        if (ib) enqueue_classify(b, s, p, sel);
+        if (low != s) {
+            cudaEventRecord(b->ev_ib, s);
+            cudaStreamWaitEvent(low, b->ev_ib, 0);
+        }
+        enqueue_sc(b, low, p, par, wa);
+        if (low != s) {
+            cudaEventRecord(b->ev_sc, low);
+            cudaStreamWaitEvent(s, b->ev_sc, 0);
+        }
+        if (ib && (!ring || k == steps - 1)) enqueue_interp(b, s, p, sel);
+        par ^= 1;
     }
-    const int grid = std::max(1, std::min(b->ntiles, b->sm_count * b->sc_blocks_per_sm));
-    launch_b_sc(b->Q, b->storage, write_all, b->any_ext, b->d_slots, b->d_tiles, b->ntiles, par,
-                grid, s);
-    if (b->nnodes > 0)
-        launch_b_ib(b->dim, b->storage, 2, b->d_slots, b->d_nodes, b->nnodes, b->d_faces,
-                    b->nfaces, s);
 }
 
 iblb_status get_graph(iblb_batch_s* b, int steps, bool last, cudaGraphExec_t* out)
@@ -894,17 +1063,22 @@ iblb_status get_graph(iblb_batch_s* b, int steps, bool last, cudaGraphExec_t* ou
         *out = it->second;
         return IBLB_OK;
     }
-    BCK(b, cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-    int par = b->par;
-    for (int k = 0; k < steps; k++) {
-        enqueue_step(b, b->cap, par, last && k == steps - 1);
-        par ^= 1;
+    BCK(b, cudaStreamBeginCapture(b->cap[0], cudaStreamCaptureModeThreadLocal));
+    if (b->parts.size() > 1) {
+        cudaEventRecord(b->ev_fork, b->cap[0]);
+        cudaStreamWaitEvent(b->cap[1], b->ev_fork, 0);
+        enqueue_steps(b, b->cap[1], b->low[1], b->parts[1], b->par, steps, last);
+        cudaEventRecord(b->ev_join, b->cap[1]);
+        enqueue_steps(b, b->cap[0], b->low[0], b->parts[0], b->par, steps, last);
+        cudaStreamWaitEvent(b->cap[0], b->ev_join, 0);
+    } else {
+        enqueue_steps(b, b->cap[0], b->cap[0], b->parts[0], b->par, steps, last);
     }
     cudaGraph_t graph;
-    cudaError_t e = cudaStreamEndCapture(b->cap, &graph);
+    cudaError_t e = cudaStreamEndCapture(b->cap[0], &graph);
     if (e != cudaSuccess) return bfail(b, IBLB_ECUDA, std::string("capture: ") + cudaGetErrorString(e));
     cudaGraphExec_t exec;
-    e = cudaGraphInstantiate(&exec, graph, 0);
+    e = cudaGraphInstantiate(&exec, graph, cudaGraphInstantiateFlagUseNodePriority);
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return bfail(b, IBLB_ECUDA, std::string("instantiate: ") + cudaGetErrorString(e));
     b->graphs[key] = exec;
@@ -1059,7 +1233,14 @@ iblb_status iblb_batch_create(int lattice, int storage, size_t hbm_budget_bytes,
     if (e == cudaSuccess) e = cudaMalloc(&b->d_slots, sizeof(SlotDev) * max_slots);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_partial, sizeof(double) * 1024);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_obs, sizeof(double) * OBS_DOUBLES);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
+    int lo = 0, hi = 0;
+    if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
+    for (int k = 0; k < 2; k++) {
+        if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->cap[k], cudaStreamNonBlocking, hi);
+        if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&b->low[k], cudaStreamNonBlocking, lo);
+    }
+    for (cudaEvent_t* ev : {&b->ev_fork, &b->ev_join, &b->ev_ib, &b->ev_sc})
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         iblb_batch_destroy(b);
         return e == cudaErrorMemoryAllocation ? IBLB_ENOMEM : IBLB_ECUDA;
@@ -1079,6 +1260,7 @@ void iblb_batch_destroy(iblb_batch b)
     cudaFree(b->d_tiles);
     cudaFree(b->d_nodes);
     cudaFree(b->d_faces);
+    cudaFree(b->d_rings);
     cudaFree(b->d_tt);
     cudaFree(b->d_detslots);
     cudaFree(b->detb.cnt);
@@ -1093,7 +1275,10 @@ void iblb_batch_destroy(iblb_batch b)
     cudaFree(b->detb.wts);
     cudaFree(b->d_partial);
     cudaFree(b->d_obs);
-    if (b->cap) cudaStreamDestroy(b->cap);
+    for (cudaStream_t st : {b->cap[0], b->cap[1], b->low[0], b->low[1]})
+        if (st) cudaStreamDestroy(st);
+    for (cudaEvent_t ev : {b->ev_fork, b->ev_join, b->ev_ib, b->ev_sc})
+        if (ev) cudaEventDestroy(ev);
     delete b;
 }
 
@@ -1179,6 +1364,7 @@ iblb_status iblb_batch_admit(iblb_batch b, const iblb_config* cfg, const double*
     d.scale = b->storage == IBLB_FP16_DEV ? std::ldexp(1.0f, sexp) : 1.0f;
     d.inv_scale = 1.0f / d.scale;
     d.q = (double*)(base + L.q);
+    d.q2 = (dim == 2 && b->elt != 2) ? (double*)(base + L.q2) : nullptr;
     d.phi = (double*)(base + L.phi);
     d.N = n_nodes;
     d.M = dim == 3 ? n_faces : n_nodes;
@@ -1303,14 +1489,19 @@ iblb_status batch_run(iblb_batch_s* b, int max_steps, int* n_completed, double* 
                     st = bfail(b, IBLB_ECUDA, std::string("graph launch: ") + cudaGetErrorString(e));
                     break;
                 }
-                b->launches += (long long)k * kernels_per_step(b);
-                add_launches((long long)k * kernels_per_step(b));
+                b->launches += graph_kernels(b, k);
+                add_launches(graph_kernels(b, k));
                 b->par ^= (k & 1);
                 done_here += k;
             }
             if (st != IBLB_OK) break;
         } else {
             const double bytes = active_stream_bytes(b);
+            Part all;
+            all.t1 = b->ntiles;
+            all.n1 = b->nnodes;
+            all.f1 = b->nfaces;
+            all.c1 = b->ntt;
             const int grid = std::max(1, std::min(b->ntiles, b->sm_count * b->sc_blocks_per_sm));
             for (int k = 0; k < seg; k++) {
                 const bool last = (k == seg - 1);
@@ -1320,8 +1511,8 @@ iblb_status batch_run(iblb_batch_s* b, int max_steps, int* n_completed, double* 
                                 b->d_faces, b->nfaces, b->stream);
                 cudaEventRecord(ev[1], b->stream);
                 if (b->nnodes > 0) {
-                    enqueue_spread(b, b->stream);
-                    enqueue_classify(b, b->stream);
+                    enqueue_spread(b, b->stream, all);
+                    enqueue_classify(b, b->stream, all);
                 }
                 cudaEventRecord(ev[2], b->stream);
                 launch_b_sc(b->Q, b->storage, last, b->any_ext, b->d_slots, b->d_tiles,

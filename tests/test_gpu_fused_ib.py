@@ -60,3 +60,59 @@ def test_default_binary16_ring_has_the_pipelined_bits(nx, ny):
         out.append(g.populations())
         g.close()
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("which", ["2d", "3d"])
+@pytest.mark.parametrize("storage,tol", [(iblb.FP64, 1e-12), (iblb.FP32_DEV, 1e-5)])
+def test_batch_in_two_parts_matches_single_engine(which, storage, tol):
+    # enough cells for two parts; the slots end at different steps, so the
+    # parts are cut anew, down to one slot in one part
+    if which == "2d":
+        wls = [small_2d(nx=nx, ny=ny, R=9.0, N=N) for nx, ny, N in ((700, 300, 61), (33, 40, 29), (260, 330, 90))]
+    else:
+        wls = [small_3d(n=n, nz=nz, R=7.0, level=2) for n, nz in ((80, 40), (24, 22), (40, 40))]
+    steps = (40, 17, 33)
+    b = iblb.Batch(wls[0].lattice, storage, 1 << 30, max_slots=4)
+    slots = [b.admit_workload(w, n_steps=n) for w, n in zip(wls, steps)]
+    b.run(64)
+    for w, n, s in zip(wls, steps, slots):
+        _, u, q = b.fields(s)
+        g = iblb.Simulation.from_workload(w, storage=storage)
+        g.step(n)
+        _, ug, qg = g.fields()
+        g.close()
+        assert np.linalg.norm(u - ug) <= tol * np.linalg.norm(ug)
+        assert np.max(np.abs(q - qg)) <= tol * 10
+    b.close()
+
+
+@pytest.mark.parametrize("which", ["2d", "3d"])
+def test_observables_over_many_blocks(which):
+    # more nodes than one block takes in a pass, against the oracle's estimator
+    import oracle
+    from paper_2604_17463_gb300 import workloads as W
+    if which == "2d":
+        wl = W.spreading_2d_2048x512(downscale=4)
+        nodes = W.truncated_circle(2000, 50.0, 150.0, W.WALL_PLANE + wl.xi, 256.0)
+        faces = None
+    else:
+        wl = small_3d(n=64, nz=48, R=15.0, level=2)
+        nodes, faces = W.icosphere(5, 15.0, (32.3, 31.8, W.WALL_PLANE + 17.0))
+    kw = dict(tau=wl.tau, sigma=wl.sigma, xi=wl.xi, theta_eq_deg=wl.theta_eq_deg)
+    g = iblb.Simulation(wl.lattice, wl.nx, wl.ny, wl.nz, **kw)
+    o = oracle.Sim(wl.lattice, wl.nx, wl.ny, wl.nz, **kw)
+    g.set_interface(nodes, faces)
+    o.set_interface(nodes, faces)
+    a, b = g.observables(), o.observables()
+    # at rest every density is 1: the mass is the number of fluid cells, exactly
+    assert a["mass"] == wl.fluid_cells
+    for k in ("volume", "height", "film", "d_min", "radius"):
+        assert np.isclose(a[k], b[k], rtol=1e-11, atol=1e-11, equal_nan=True), k
+    # the whole sphere meets the plane of its lowest node at 180 degrees, where
+    # the angle and the contact radius are the square roots of rounding errors:
+    # their cosine and square are compared
+    assert np.isclose(np.cos(np.radians(a["theta_deg"])), np.cos(np.radians(b["theta_deg"])), rtol=0, atol=1e-11)
+    assert np.isclose(a["r_cl"] ** 2, b["r_cl"] ** 2, rtol=0, atol=1e-11 * b["radius"] ** 2)
+    assert np.allclose(a["centre"], b["centre"], rtol=1e-11, atol=1e-11)
+    g.close()
+    o.close()
