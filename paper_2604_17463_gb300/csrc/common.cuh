@@ -326,8 +326,11 @@ void launch_observables(int dim, const double* q, int N, const int* tri, int M,
 // f = f_eq(rho, u) in storage form (deviation from w, scaled); rho may be null (1).
 void launch_set_equilibrium(int Q, int storage, int dim, const double* rho, const double* u,
                             void* dst, long long ncell, float scale, cudaStream_t s);
-// Deformation index of the interface in the shear plane: out[5] =
-// {D, r1, r3, inclination (deg), enclosed area / volume}.
+// Deformation index of the interface in the shear plane: the first 5 of the
+// DEFORMATION_DOUBLES doubles of out = {D, r1, r3, inclination (deg), enclosed
+// area / volume}, the rest workspace.
+constexpr int DEFORMATION_DOUBLES = 16 + 9 * OBS_GRID;
+constexpr int DEFORMATION_KERNELS = 3;
 void launch_deformation(int dim, const double* q, int N, const int* tri, int M, double* out,
                         cudaStream_t s);
 

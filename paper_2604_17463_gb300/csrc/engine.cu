@@ -71,7 +71,7 @@ struct iblb_sim {
     int* csr_ptr = nullptr;
     int* entry_pos = nullptr;    // CSR position of each (face, corner) (3D)
     double* entry_rec = nullptr; // per-(face, corner) geometry records in CSR order (3D)
-    double* defo = nullptr;      // deformation output [8]
+    double* defo = nullptr;      // deformation output and workspace
     double* eref = nullptr;      // elastic reference of the interface (shear_modulus != 0)
     unsigned* rng = nullptr;     // two-entry step counter (binary16 stochastic rounding)
     bool moving = false;         // walls with a tangential velocity
@@ -575,7 +575,7 @@ iblb_status iblb_create(const iblb_config* cfg, void* cuda_stream, iblb_handle* 
     if ((e = cudaMalloc(&h->partial, sizeof(double) * h->npartial)) != cudaSuccess)
         return bail(e, "partial");
     if ((e = cudaMalloc(&h->obs, sizeof(double) * OBS_DOUBLES)) != cudaSuccess) return bail(e, "obs");
-    if ((e = cudaMalloc(&h->defo, sizeof(double) * 8)) != cudaSuccess) return bail(e, "obs");
+    if ((e = cudaMalloc(&h->defo, sizeof(double) * DEFORMATION_DOUBLES)) != cudaSuccess) return bail(e, "obs");
     if ((e = cudaMalloc(&h->rng, sizeof(unsigned) * 2)) != cudaSuccess) return bail(e, "obs");
     cudaMemsetAsync(h->rng, 0, sizeof(unsigned) * 2, h->stream);
     if (h->two_tau) {
@@ -1044,7 +1044,7 @@ iblb_status iblb_deformation(iblb_handle h, double* out)
     if (h->N < 3 || (h->dim == 3 && h->M < 4))
         return fail(h, IBLB_EINVAL, "deformation needs a closed interface");
     launch_deformation(h->dim, h->q, h->N, h->tri, h->M, h->defo, h->stream);
-    g_launches++;
+    g_launches += DEFORMATION_KERNELS;
     CK(h, cudaGetLastError());
     CK(h, cudaMemcpyAsync(out, h->defo, sizeof(double) * 5, cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));

@@ -223,7 +223,6 @@ void launch_interp(int storage, int dim, double* q, const void* moments, int N, 
 // deterministic.  Contact-angle estimator: algebraic least-squares circle
 // (2D) / sphere (3D) through the nodes with d > 3 xi, centred on their mean,
 // intersected with the plane d = min_j d_j.
-constexpr int OBS_BLOCK = 1024;
 
 // Reduce nv values per thread to thread 0 (sum), in a fixed order.
 template <int B>
@@ -522,26 +521,36 @@ __global__ void __launch_bounds__(32) k_obs_last(ObsArgs a, int grid)
 // int x x^T = |K| (sum v_k v_k^T + s s^T) / ((d + 1)(d + 2)), s = sum v_k.
 // The central second moments in the shear plane (x and the wall axis) give
 // the semi-axes sqrt(4 lambda / area) (2D) or sqrt(5 lambda / volume) (3D).
-__global__ void __launch_bounds__(OBS_BLOCK)
-k_deformation(int dim, const double* __restrict__ q, int N, const int* __restrict__ tri, int M,
-              double* out)
+// Three kernels: node sums, simplex sums about their mean, results; up to
+// OBS_GRID blocks (the call with 20 480 faces took 0.49 ms in one block, so 0.06).
+__global__ void __launch_bounds__(OBS_THREADS) k_def_mean(int dim, const double* __restrict__ q, int N, double* part)
 {
-    __shared__ double sh[6][OBS_BLOCK / 32];
-    __shared__ double p0s[3];
-    const int t = threadIdx.x;
-    const int w = dim - 1;
-    double v[6];
-    for (int k = 0; k < 6; k++) v[k] = 0.0;
-    for (int j = t; j < N; j += OBS_BLOCK)
+    __shared__ double sh[3][OBS_THREADS / 32];
+    double v[3] = {0, 0, 0};
+    for (int j = blockIdx.x * OBS_THREADS + threadIdx.x; j < N; j += gridDim.x * OBS_THREADS)
         for (int k = 0; k < dim; k++) v[k] += q[dim * j + k];
-    block_sum<OBS_BLOCK>(v, 3, sh);
-    if (t == 0)
-        for (int k = 0; k < 3; k++) p0s[k] = k < dim ? v[k] / N : 0.0;
+    block_sum<OBS_THREADS>(v, 3, sh);
+    if (threadIdx.x == 0)
+        for (int k = 0; k < 3; k++) part[3 * blockIdx.x + k] = v[k];
+}
+
+__global__ void __launch_bounds__(OBS_THREADS)
+k_def_moments(int dim, const double* __restrict__ q, int N, const int* __restrict__ tri, int M,
+              const double* __restrict__ mean_part, double* part)
+{
+    __shared__ double sh[6][OBS_THREADS / 32];
+    __shared__ double p0s[3];
+    if (threadIdx.x < 32)
+        for (int k = 0; k < 3; k++) {
+            const double s = column_sum(mean_part, 3, k, gridDim.x);
+            if (threadIdx.x == 0) p0s[k] = k < dim ? s / N : 0.0;
+        }
     __syncthreads();
     const double p0[3] = {p0s[0], p0s[1], p0s[2]};
-    for (int k = 0; k < 6; k++) v[k] = 0.0;
+    const int w = dim - 1;
+    double v[6] = {0, 0, 0, 0, 0, 0};
     const int nsimp = dim == 2 ? N : M;
-    for (int e = t; e < nsimp; e += OBS_BLOCK) {
+    for (int e = blockIdx.x * OBS_THREADS + threadIdx.x; e < nsimp; e += gridDim.x * OBS_THREADS) {
         double a[3] = {0, 0, 0}, b[3] = {0, 0, 0}, c[3] = {0, 0, 0};
         double meas;
         if (dim == 2) {
@@ -572,8 +581,16 @@ k_deformation(int dim, const double* __restrict__ q, int N, const int* __restric
         v[4] += f2 * (a[w] * a[w] + b[w] * b[w] + c[w] * c[w] + sw * sw);
         v[5] += f2 * (a[0] * a[w] + b[0] * b[w] + c[0] * c[w] + sx * sw);
     }
-    block_sum<OBS_BLOCK>(v, 6, sh);
-    if (t == 0) {
+    block_sum<OBS_THREADS>(v, 6, sh);
+    if (threadIdx.x == 0)
+        for (int k = 0; k < 6; k++) part[6 * blockIdx.x + k] = v[k];
+}
+
+__global__ void __launch_bounds__(32) k_def_last(int dim, const double* __restrict__ part, int grid, double* out)
+{
+    double v[6];
+    for (int k = 0; k < 6; k++) v[k] = column_sum(part, 6, k, grid);
+    if (threadIdx.x == 0) {
         const double vol = v[0];
         const double gx = v[1] / vol, gw = v[2] / vol;
         const double sxx = v[3] - vol * gx * gx;
@@ -594,7 +611,15 @@ k_deformation(int dim, const double* __restrict__ q, int N, const int* __restric
 void launch_deformation(int dim, const double* q, int N, const int* tri, int M, double* out,
                         cudaStream_t s)
 {
-    k_deformation<<<1, OBS_BLOCK, 0, s>>>(dim, q, N, tri, M, out);
+    const int n = dim == 2 ? N : (M > N ? M : N);
+    int grid = (n + OBS_THREADS - 1) / OBS_THREADS;
+    grid = grid < 1 ? 1 : (grid > OBS_GRID ? OBS_GRID : grid);
+    double* mean_part = out + 16;
+    double* part = mean_part + 3 * OBS_GRID;
+    static_assert(16 + 9 * OBS_GRID <= DEFORMATION_DOUBLES, "deformation workspace");
+    k_def_mean<<<grid, OBS_THREADS, 0, s>>>(dim, q, N, mean_part);
+    k_def_moments<<<grid, OBS_THREADS, 0, s>>>(dim, q, N, tri, M, mean_part, part);
+    k_def_last<<<1, 32, 0, s>>>(dim, part, grid, out);
 }
 
 void launch_observables(int dim, const double* q, int N, const int* tri, int M,
