@@ -119,3 +119,23 @@ def test_observables_over_many_blocks(which):
     assert np.allclose(a["centre"], b["centre"], rtol=1e-11, atol=1e-11)
     g.close()
     o.close()
+
+
+@pytest.mark.parametrize("heap", [31, 33, 200, 300])
+def test_ordered_spread_sorts_crowded_bins(heap):
+    # `heap` nodes of a ring within one bin of the ordered spread: the force
+    # field is that of the atomic spread up to the order of the additions, and
+    # the same twice
+    import math
+    n = heap + 60
+    a = np.concatenate([np.linspace(-0.02, 0.02, heap, endpoint=False),
+                        np.linspace(0.02, 2 * math.pi - 0.02, 60, endpoint=False)])
+    nodes = np.stack([32.4 + 12 * np.cos(a), 16.3 + 12 * np.sin(a)], axis=1)
+    out = []
+    for ordered in (True, True, False):
+        g = iblb.Simulation(iblb.D2Q9, 64, 40, wetting=False, sigma=1e-3, deterministic_spread=ordered)
+        g.set_interface(nodes)
+        out.append(g.force_field())
+        g.close()
+    assert np.array_equal(out[0], out[1])
+    assert np.max(np.abs(out[0] - out[2])) <= 1e-12 * np.max(np.abs(out[2]))
