@@ -299,7 +299,8 @@ typedef struct {
                                      iblb_autotune. */
     int step_overlap;             /* iblb_step with an interface: 0 (default)
                                      overlaps on 3D lattices of at least 2^20
-                                     cells, 1 always, 2 never.  Overlapped, a
+                                     cells (FP64: 2^15), 1 always, 2 never.
+                                     Overlapped, a
                                      step runs the stream-collide of every
                                      cell with the body force only on one
                                      stream while the nodal forces are

@@ -141,13 +141,17 @@ int spread_kernels(const iblb_sim* h) { return h->det ? DET_KERNELS : 1; }
 bool use_groups(const iblb_sim* h) { return h->grouped && h->tune.ib_grouped; }
 int regroup_kernels(const iblb_sim* h) { return use_groups(h) ? REGROUP_KERNELS : 0; }
 // The overlapped step (enqueue_step_overlapped): with an interface, and
-// (automatic mode) on a 3D lattice of at least 2^20 cells.
-// A 2D ring's IB kernels are too short to hide: on the 2048 x 512 spreading
-// drop the overlapped step measured 25.5 us against 21.5 us serial.
+// (automatic mode) on a 3D lattice of at least 2^20 cells, in FP64 of at least
+// 2^15.  Below that the IB kernels of an FP32 step are too short to hide behind
+// the bulk pass and pay for the band pass: 101 x 101 x 77 50.2 us serial, 49.9
+// overlapped, 64 x 64 x 40 25.3 and 25.8; FP64 64 x 64 x 40 88.8 and 73.9,
+// 96 x 96 x 72 216 and 202, 40 x 40 x 32 71.1 and 64.3.  A 2D ring's are
+// shorter still (2048 x 512 spreading drop: 21.5 us serial, 25.5 overlapped).
 bool overlapped(const iblb_sim* h)
 {
     if (h->N == 0 || h->tune.step_overlap == 2) return false;
-    return h->tune.step_overlap == 1 || (h->dim == 3 && h->g.ncell >= (1LL << 20));
+    const long long least = h->storage == IBLB_FP64 ? 1LL << 15 : 1LL << 20;
+    return h->tune.step_overlap == 1 || (h->dim == 3 && h->g.ncell >= least);
 }
 // The serial step of a ring with one fused IB kernel per step (k_ring);
 // the ordered spread and the overlapped step keep their separate kernels, and
