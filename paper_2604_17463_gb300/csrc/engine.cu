@@ -61,7 +61,8 @@ struct iblb_sim {
     int* err = nullptr;
     double* partial = nullptr;
     int npartial = 0;
-    double* obs = nullptr;     // OBS_DOUBLES
+    double* obs = nullptr;     // 12 doubles
+    double* obs_ws = nullptr;  // workspace of observables and deformation, from the first call on
     // interface
     int N = 0, M = 0;
     double* q = nullptr;         // node positions
@@ -71,7 +72,7 @@ struct iblb_sim {
     int* csr_ptr = nullptr;
     int* entry_pos = nullptr;    // CSR position of each (face, corner) (3D)
     double* entry_rec = nullptr; // per-(face, corner) geometry records in CSR order (3D)
-    double* defo = nullptr;      // deformation output and workspace
+    double* defo = nullptr;      // deformation output [8]
     double* eref = nullptr;      // elastic reference of the interface (shear_modulus != 0)
     unsigned* rng = nullptr;     // two-entry step counter (binary16 stochastic rounding)
     bool moving = false;         // walls with a tangential velocity
@@ -578,8 +579,8 @@ iblb_status iblb_create(const iblb_config* cfg, void* cuda_stream, iblb_handle* 
     h->npartial = mass_partial_blocks(g);
     if ((e = cudaMalloc(&h->partial, sizeof(double) * h->npartial)) != cudaSuccess)
         return bail(e, "partial");
-    if ((e = cudaMalloc(&h->obs, sizeof(double) * OBS_DOUBLES)) != cudaSuccess) return bail(e, "obs");
-    if ((e = cudaMalloc(&h->defo, sizeof(double) * DEFORMATION_DOUBLES)) != cudaSuccess) return bail(e, "obs");
+    if ((e = cudaMalloc(&h->obs, sizeof(double) * 12)) != cudaSuccess) return bail(e, "obs");
+    if ((e = cudaMalloc(&h->defo, sizeof(double) * 8)) != cudaSuccess) return bail(e, "obs");
     if ((e = cudaMalloc(&h->rng, sizeof(unsigned) * 2)) != cudaSuccess) return bail(e, "obs");
     cudaMemsetAsync(h->rng, 0, sizeof(unsigned) * 2, h->stream);
     if (h->two_tau) {
@@ -670,6 +671,7 @@ void iblb_destroy(iblb_handle h)
     free_dev(h->err);
     free_dev(h->partial);
     free_dev(h->obs);
+    free_dev(h->obs_ws);
     free_dev(h->q);
     free_dev(h->q2);
     free_dev(h->phi);
@@ -759,7 +761,7 @@ iblb_status iblb_set_interface(iblb_handle h, const double* xyz, int n_nodes, co
     if (n_nodes == 0) return IBLB_OK;
     const size_t qb = sizeof(double) * (size_t)n_nodes * dim;
     CK(h, cudaMalloc(&h->q, qb));
-    if (dim == 2) CK(h, cudaMalloc(&h->q2, qb));
+    if (dim == 2 && h->storage != IBLB_FP16_DEV) CK(h, cudaMalloc(&h->q2, qb));
     CK(h, cudaMalloc(&h->phi, qb));
     CK(h, cudaMemcpyAsync(h->q, xyz, qb, cudaMemcpyHostToDevice, h->stream));
     if (h->det) {
@@ -912,10 +914,11 @@ iblb_status iblb_get_populations(iblb_handle h, double* f)
 iblb_status iblb_observables(iblb_handle h, iblb_obs* out)
 {
     if (!h || !out) return IBLB_EINVAL;
+    if (!h->obs_ws) CK(h, cudaMalloc(&h->obs_ws, sizeof(double) * OBS_WS));
     launch_mass_partials(h->Q, h->storage, h->f[h->cur], h->g, h->sp.inv_scale, h->partial,
                          h->stream);
     launch_observables(h->dim, h->q, h->N, h->tri, h->M, h->partial, h->npartial, h->cfg.xi, 0.5,
-                       h->obs, h->stream);
+                       h->obs, h->obs_ws, h->stream);
     g_launches += 1 + OBS_KERNELS;
     CK(h, cudaGetLastError());
     double v[12];
@@ -1047,7 +1050,8 @@ iblb_status iblb_deformation(iblb_handle h, double* out)
     if (!h || !out) return IBLB_EINVAL;
     if (h->N < 3 || (h->dim == 3 && h->M < 4))
         return fail(h, IBLB_EINVAL, "deformation needs a closed interface");
-    launch_deformation(h->dim, h->q, h->N, h->tri, h->M, h->defo, h->stream);
+    if (!h->obs_ws) CK(h, cudaMalloc(&h->obs_ws, sizeof(double) * OBS_WS));
+    launch_deformation(h->dim, h->q, h->N, h->tri, h->M, h->defo, h->obs_ws, h->stream);
     g_launches += DEFORMATION_KERNELS;
     CK(h, cudaGetLastError());
     CK(h, cudaMemcpyAsync(out, h->defo, sizeof(double) * 5, cudaMemcpyDeviceToHost, h->stream));

@@ -609,14 +609,14 @@ __global__ void __launch_bounds__(32) k_def_last(int dim, const double* __restri
 }
 
 void launch_deformation(int dim, const double* q, int N, const int* tri, int M, double* out,
-                        cudaStream_t s)
+                        double* ws, cudaStream_t s)
 {
     const int n = dim == 2 ? N : (M > N ? M : N);
     int grid = (n + OBS_THREADS - 1) / OBS_THREADS;
     grid = grid < 1 ? 1 : (grid > OBS_GRID ? OBS_GRID : grid);
-    double* mean_part = out + 16;
+    double* mean_part = ws;
     double* part = mean_part + 3 * OBS_GRID;
-    static_assert(16 + 9 * OBS_GRID <= DEFORMATION_DOUBLES, "deformation workspace");
+    static_assert(9 * OBS_GRID <= OBS_WS, "deformation workspace");
     k_def_mean<<<grid, OBS_THREADS, 0, s>>>(dim, q, N, mean_part);
     k_def_moments<<<grid, OBS_THREADS, 0, s>>>(dim, q, N, tri, M, mean_part, part);
     k_def_last<<<1, 32, 0, s>>>(dim, part, grid, out);
@@ -624,13 +624,13 @@ void launch_deformation(int dim, const double* q, int N, const int* tri, int M, 
 
 void launch_observables(int dim, const double* q, int N, const int* tri, int M,
                         const double* mass_partial, int n_partial, double xi, double wall_plane,
-                        double* out, cudaStream_t s)
+                        double* out, double* ws, cudaStream_t s)
 {
     ObsArgs a{dim, q, N, tri, M, mass_partial, n_partial, xi, wall_plane, out, nullptr, nullptr, nullptr};
-    a.p1 = out + 16;
+    a.p1 = ws;
     a.p2 = a.p1 + OBS_P1 * OBS_GRID;
     a.p3 = a.p2 + OBS_P2 * OBS_GRID;
-    static_assert(16 + (OBS_P1 + OBS_P2 + OBS_P3) * OBS_GRID <= OBS_DOUBLES, "observables workspace");
+    static_assert((OBS_P1 + OBS_P2 + OBS_P3) * OBS_GRID <= OBS_WS, "observables workspace");
     int grid = ((N > n_partial ? N : n_partial) + OBS_THREADS - 1) / OBS_THREADS;
     grid = grid < 1 ? 1 : (grid > OBS_GRID ? OBS_GRID : grid);
     k_obs_sums<<<grid, OBS_THREADS, 0, s>>>(a);
