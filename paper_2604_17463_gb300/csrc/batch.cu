@@ -72,16 +72,18 @@ constexpr int BT = 128;  // threads per stream-collide block
 // (their loads are all issued before any of them is collided, so that
 // enough bytes are in flight per SM for the HBM bound), and the resident
 // blocks per SM asked of the register allocator; chosen by measurement on
-// the 256-drop set (D2Q9 FP32: 3 segments at 5 blocks beat 2 at 6 or 8 and
-// 4 at 4; D2Q9 binary16: 2 at 6) and on 40 D3Q19 requests of the serving
-// mix (FP32: 2 segments at 4 blocks with the next item prefetched, 1.89 ms
-// per launch, beat 1 segment at 5, 6, 7 or 8 blocks, 2.99-3.71 ms, and 2 at
-// 3 blocks, 1.96 ms; binary16: 2 at 4, 1.63 ms, beat 1 at 6 or 8, 2.5 ms).
-// FP64 is bound by its arithmetic.  A slot's work items hold cpt segments,
-// a multiple of this.
+// the 256-drop set (D2Q9 FP32, us per launch: 2 segments at 6 blocks 172, at 5
+// 179, 3 at 5 207, 3 at 4 214, 4 at 4 176; before the collision left the zero
+// components out, 3 at 5 took 175; D2Q9 binary16: 2 at 6) and on 40 D3Q19
+// requests of the serving mix (FP32: 2 segments at 4 blocks with the next item
+// prefetched, 1.89 ms per launch, beat 1 segment at 5, 6, 7 or 8 blocks,
+// 2.99-3.71 ms, and 2 at 3 blocks, 1.96 ms; binary16: 2 at 4, 1.63 ms, beat 1 at
+// 6 or 8, 2.5 ms).  FP64 is bound by its arithmetic (the 256 drops: 2400 us with
+// the force terms in every cell, now 1675).  A slot's work items hold cpt
+// segments, a multiple of this.
 constexpr int b_ilp_of(int Q, int ST)
 {
-    return ST == ST_FP64 ? 1 : (Q == 9 ? (ST == ST_FP32 ? 3 : 2) : 2);
+    return ST == ST_FP64 ? 1 : 2;
 }
 template <int Q, int ST> struct BIlp {
     static constexpr int value = b_ilp_of(Q, ST);
@@ -89,7 +91,7 @@ template <int Q, int ST> struct BIlp {
 int b_ilp(int Q, int storage) { return b_ilp_of(Q, storage); }
 
 template <int Q, int ST> struct BMinBlocks {
-    static constexpr int value = ST == ST_FP64 ? (Q == 9 ? 5 : 4) : (Q == 9 ? (ST == ST_FP32 ? 5 : 6) : 4);
+    static constexpr int value = ST == ST_FP64 ? (Q == 9 ? 5 : 4) : (Q == 9 ? 6 : 4);
 };
 // The next work item is loaded while the current one is processed (D3Q19
 // FP32; measured slower for binary16).
