@@ -342,8 +342,8 @@ long long iblb_fluid_cells(iblb_handle h);
  * at a time, and each slot computes exactly the step of iblb_step (Sec. 2,
  * Eq. 1-11 and forward Euler).  A batch advances many independent droplet simulations ("slots") of one
  * lattice type and one storage form with shared launches: every phase of a
- * time step is one launch over all active slots (the stream-collide phase a
- * persistent kernel walking a (slot, tile) work list).  Slot state lives in
+ * time step is one launch over all active slots (3D: over each half of them;
+ * the stream-collide phase walks a (slot, tile) work list).  Slot state lives in
  * one device arena of hbm_budget_bytes allocated at creation; a request is
  * admitted when its footprint fits (first fit), else IBLB_EAGAIN.  Slots
  * must have walls, no body force, and the batch's lattice and storage; the

@@ -4,12 +4,14 @@
 // A batch holds simulations ("slots") of one lattice type and one population
 // storage form.  Each time step runs the same phases as a single simulation
 // (nodal forces, spread, stream-collide, interpolate + advect; Sec. 2 of the
-// paper), but every phase is ONE launch over all active slots:
+// paper), but a phase is ONE launch over many slots:
 //   - stream-collide: a persistent kernel whose warps walk contiguous ranges
 //     of a (slot, row, x0) work list; an item is cpt 32-cell segments of one
 //     lattice row of one slot, cpt chosen per slot by the tile autotuner;
-//   - IB phases: one thread (forces) or one warp (spread, interpolation) per
-//     (slot, node) item of a concatenated node list.
+//   - IB phases: FP64 and FP32 rings in one kernel, a warp per 30 nodes
+//     (k_b_ring); meshes a thread per face, then per node (force and spread),
+//     then per node (interpolation); binary16 rings and the ordered spread one
+//     kernel per phase.  Meshes step in two parts on two streams (Part).
 // Slot state lives in one device arena (the batch's HBM budget) carved by a
 // first-fit allocator; a request is admitted when its footprint fits, else
 // the call returns IBLB_EAGAIN.  Slots advance together; a run stops at each
