@@ -46,9 +46,8 @@ __device__ __forceinline__ float delta4f(float r)
 // s = sqrt(1 + 4 fr - 4 fr^2), so one root serves the four weights.
 // The IB kernels are chains of dependent operations on few warps (FP64 issues
 // 2 lanes per clock and SM): against one root per weight, with the two
-// branches of the kernel diverging in the warp, the step of the FP64 128 x 64
-// ring (213 nodes) went from 34.7 to 25.4 us, of the FP32 2048 x 512 one
-// (2000 nodes) from 27.6 to 24.8 us.
+// branches of the kernel diverging in the warp, and with one-warp blocks, the
+// step of the FP64 128 x 64 ring (213 nodes) went from 34.7 to 25.4 us.
 //
 // 2D interfaces in FP32 keep one root per weight (cheap there): the ring's
 // forces then round as they always have, and a binary16 run, whose stochastic
