@@ -255,7 +255,10 @@ enum {
  * bucket is 0.  Synchronises. */
 iblb_status iblb_step_profiled(iblb_handle h, int n_steps, double* kernel_ms);
 
-/* Launch shape of the stream-collide kernel (results do not depend on it).
+/* Launch shape of the stream-collide kernel.  Results do not depend on the
+ * sizes of a variant; two variants round some sums differently (FP64, FP32: in
+ * the last bits; binary16: another realisation of the stochastic rounding),
+ * but for D2Q9 with binary16 storage, where variants 0 and 1 give the same bits.
  *   variant 0: the plain kernel, one cell per thread, block_x threads per
  *              block along x (64, 128 or 256), evict-first stores of the new
  *              populations when streaming_stores != 0;

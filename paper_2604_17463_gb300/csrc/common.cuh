@@ -83,6 +83,7 @@ struct StreamParams {
     float omega_f;         // the same in FP32 (no per-thread conversion on the FP32 paths)
     float body_f[3];
     int has_body;          // any component of the body force is not zero
+    int rest_fused;        // D2Q9 binary16: see cell_update_h9
     // viscosity ratio: cells outside the interface relax with omega_out
     int two_tau;
     double omega_out;
@@ -141,7 +142,6 @@ struct Tuning {
     long long wait_limit = 0;   // pipelined kernel: clock cycles a wait may take (0: ~2 s)
     int ib_grouped = 0;         // 3D interfaces: 1 spreads / interpolates by spatial groups of
                                 // nodes (ib_groups.cu) instead of one thread per node
-    int pipe_form = 0;          // plain kernel, D2Q9 binary16: the pipelined kernel's bits
     int step_overlap = 0;       // 0: overlapped step on 3D lattices of >= 2^20 cells; 1: always;
                                 // 2: never (see enqueue_step_overlapped)
 };

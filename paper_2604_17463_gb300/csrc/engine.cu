@@ -417,7 +417,7 @@ double wetting_amplitude(const iblb_config& c)
 // they hide.  Whole steps, us, pipelined against the chosen shape:
 //   D2Q9  FP64   128 x 64   22.7  18.7 (plain, 64)   2048 x 512  162  156
 //         FP32  2048 x 512  24.3  18.1 (x pairs)     512 x 128   15.6  11.2 (plain)
-//         binary16 1024 x 256  17.6  13.7 (plain, with the pipelined kernel's bits)
+//         binary16 1024 x 256  17.6  13.7 (plain)
 //   D3Q19 FP32   96 x 96 x 64  56  45 (plain, 128)   160 x 160 x 96  117  94
 //         FP64   96 x 96 x 72  640  623 (plain, 128)
 // D2Q9 FP32: x pairs need an even width and win from about 2^19 cells (1000 x
@@ -425,16 +425,12 @@ double wetting_amplitude(const iblb_config& c)
 Tuning default_tuning(const iblb_sim* h)
 {
     Tuning t;
-    PipeShape ps{};
-    const bool pipe = pipe_shape(h->Q, h->storage, h->g, h->sm_count, h->smem, t.rows_per_tile,
-                                 t.ctas_per_sm, t.consumer_warps, ps);
     if (h->dim == 3 && h->storage != IBLB_FP64 && h->g.ncell >= (1LL << 22)) return t;
     t.variant = 0;
     if (h->dim == 2 && h->storage == IBLB_FP64) t.block_x = 64;
     if (h->dim == 2 && h->storage == IBLB_FP32_DEV && pair_kernel_ok(h->storage, h->g) &&
         h->g.ncell >= (1LL << 19))
         t.variant = 2;
-    if (h->dim == 2 && h->storage == IBLB_FP16_DEV && pipe) t.pipe_form = 1;
     return t;
 }
 
@@ -653,6 +649,13 @@ iblb_status iblb_create(const iblb_config* cfg, void* cuda_stream, iblb_handle* 
         return bail(e, "shared memory limits");
     if ((e = prepare_stream_collide_pipe(h->smem)) != cudaSuccess) return bail(e, "pipe attributes");
     h->sm_count = sms;
+    // walls that move and a viscosity ratio always run the plain kernel
+    if (h->Q == 9 && h->storage == IBLB_FP16_DEV && !h->moving && !h->two_tau) {
+        const Tuning t;
+        PipeShape ps{};
+        sp.rest_fused = pipe_shape(h->Q, h->storage, g, sms, h->smem, t.rows_per_tile, t.ctas_per_sm,
+                                   t.consumer_warps, ps);
+    }
     apply_tuning(h, default_tuning(h));
     if ((e = cudaGetLastError()) != cudaSuccess) return bail(e, "init");
     *out = h;

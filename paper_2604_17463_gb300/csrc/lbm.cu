@@ -29,10 +29,7 @@ namespace iblb {
 // band != 0: the force density of the cell is added (and cleared) and the
 // moments written.  Shared by the plain kernel and the band-cell kernel of
 // the overlapped step.
-// PF (D2Q9, binary16): the products and sums are fused as the pipelined kernel
-// fuses them, so that its populations are reproduced bit for bit (the plain
-// form differs in last bits, which the stochastic rounding amplifies).
-template <int Q, int ST, bool WRITE_ALL, bool CS, bool EXT, bool BULK = false, bool PF = false>
+template <int Q, int ST, bool WRITE_ALL, bool CS, bool EXT, bool BULK = false>
 __device__ __forceinline__ void sc_cell(const typename StorageT<ST>::S* __restrict__ fin,
                                         typename StorageT<ST>::S* __restrict__ fout,
                                         typename StorageT<ST>::R* __restrict__ mom,
@@ -169,12 +166,8 @@ __device__ __forceinline__ void sc_cell(const typename StorageT<ST>::S* __restri
     constexpr int FM = force_mode<R, BULK>();
     const bool force = band || p.has_body;  // uniform in the warp
     if constexpr (D == 2) {
-        if constexpr (ST == ST_FP16 && PF) {
-            mo = cell_update<Q, R, FM>(g, force, om, Fx, Fy, Fz, (R)p.inv_scale, (R)p.scale);
-            store_cell32<Q, ST, CS>(fout, nc, c32, g, 1.0f, sr_seed(step, cell));
-        } else if constexpr (ST == ST_FP16) {
-            mo = cell_moments<Q, R, !BULK>(g, Fx, Fy, Fz, (R)p.inv_scale);
-            cell_collide<Q, R, !BULK>(g, mo, om, Fx, Fy, Fz, (R)p.scale);
+        if constexpr (ST == ST_FP16) {
+            mo = cell_update_h9<!BULK>(g, p.rest_fused, om, Fx, Fy, p.inv_scale, p.scale);
             store_cell32<Q, ST, CS>(fout, nc, c32, g, 1.0f, sr_seed(step, cell));
         } else {
             mo = cell_update<Q, R, FM>(g, force, om, Fx, Fy, Fz);
@@ -196,8 +189,7 @@ __device__ __forceinline__ void sc_cell(const typename StorageT<ST>::S* __restri
 // flags == nullptr: every cell takes the body force only (the bulk pass of
 // the overlapped step; the band cells are redone by k_band_sc).  BULK: the
 // same, with no body force either.
-template <int Q, int ST, bool WRITE_ALL, int BLOCK, bool CS, bool EXT = false, bool BULK = false,
-          bool PF = false>
+template <int Q, int ST, bool WRITE_ALL, int BLOCK, bool CS, bool EXT = false, bool BULK = false>
 __global__ void __launch_bounds__(BLOCK)
 k_stream_collide(const typename StorageT<ST>::S* __restrict__ fin,
                  typename StorageT<ST>::S* __restrict__ fout,
@@ -228,7 +220,7 @@ k_stream_collide(const typename StorageT<ST>::S* __restrict__ fin,
         step = sr_step(p.rng_in, p.rng_out,
                        blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0);
     if (x >= p.g.nx) return;
-    sc_cell<Q, ST, WRITE_ALL, CS, EXT, BULK, PF>(fin, fout, mom, F, p, x, y, z, band, step);
+    sc_cell<Q, ST, WRITE_ALL, CS, EXT, BULK>(fin, fout, mom, F, p, x, y, z, band, step);
     if (lane == 0 && band) flags[seg] = 0;
 }
 
@@ -301,20 +293,6 @@ static void launch_sc_t(bool write_all, const void* fin, void* fout, void* mom, 
         return;
     }
     const bool cs = tu.streaming_stores != 0;
-    if constexpr (Q == 9 && ST == ST_FP16) {
-        if (tu.pipe_form) {
-            dim3 grid((p.g.nx + 127) / 128, p.g.ny - 2 * (p.g.walls ? 1 : 0));
-            auto* a = (const __half*)fin;
-            auto* b = (__half*)fout;
-            if (write_all)
-                k_stream_collide<9, ST_FP16, true, 128, false, false, false, true>
-                    <<<grid, 128, 0, s>>>(a, b, (float*)mom, (float*)F, flags, p);
-            else
-                k_stream_collide<9, ST_FP16, false, 128, false, false, false, true>
-                    <<<grid, 128, 0, s>>>(a, b, (float*)mom, (float*)F, flags, p);
-            return;
-        }
-    }
     switch (tu.block_x) {
         case 64:
             if (cs) launch_sc_b<Q, ST, 64, true>(write_all, fin, fout, mom, F, flags, p, s);
