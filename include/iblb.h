@@ -106,7 +106,7 @@ typedef struct {
 } iblb_config;
 
 typedef struct {
-    double mass;          /* sum of rho over fluid cells (FP64) */
+    double mass;          /* sum of rho over fluid cells, to FP64 rounding */
     double volume;        /* enclosed area (2D) / volume (3D) of the interface */
     double height;        /* max - min node coordinate along the wall axis */
     double theta_deg;     /* apparent contact angle of the circle/sphere fit */
@@ -437,7 +437,7 @@ int iblb_batch_slot_tile(iblb_batch b, int slot);
  *
  * The paper has no counterpart: this is a service of the library.
  *
- * iblb_mass_static computes the same FP64 mass as iblb_observables (sum of
+ * iblb_mass_static computes the mass of iblb_observables, to FP64 rounding (sum of
  * rho over the fluid cells) for a population array the caller owns, without
  * allocating device memory.  It is meant for callers that cannot call
  * cudaMalloc when they need the number: a process that reserves all of its

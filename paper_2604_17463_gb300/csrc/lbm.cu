@@ -1251,12 +1251,14 @@ int mass_partial_blocks(const GridParams& g)
 }
 
 // FP32 and binary16 populations of a cell are added as an unevaluated sum of
-// two FP32 numbers (Knuth's two-sum: the rounding error of every addition is
-// found exactly and carried along), so that a cell costs three FP64 operations
-// instead of 19 conversions and 20 additions, each 16 clocks of an SM's pipe
-// per warp.  The sum is good to 2^-47 of the largest population; the FP64 sum
-// over the cells that it enters rounds at 2^-53 of the cells' number.
-// The observables call on 256 x 256 x 128 in FP32: 0.79 -> 0.26 ms.
+// three FP32 numbers: Knuth's two-sum finds the rounding error of every
+// addition exactly, and the errors are added in the same way.  What is lost are
+// the roundings of the third number, each 2^-24 of a number that is at most
+// (18 * 2^-24)^2 of the populations' absolute sum A: below 2^-59 A in all, less
+// than the one FP64 rounding that joins the three, so no FP64 sum of the
+// populations is closer.  A cell costs six FP64 operations instead of 19
+// conversions and 20 additions, each 16 clocks of an SM's pipe per warp.
+// The observables call on 256 x 256 x 128 in FP32: 0.79 -> 0.27 ms.
 template <int Q, int ST>
 __device__ __forceinline__ double cell_deviation(const typename StorageT<ST>::S* __restrict__ f,
                                                  long long nc, long long c, float inv_scale)
@@ -1270,14 +1272,17 @@ __device__ __forceinline__ double cell_deviation(const typename StorageT<ST>::S*
         for (int i = 0; i < Q; i++) dev += g[i];
         return dev;
     } else {
-        float s = g[0], e = 0.0f;
+        float s = g[0], e = 0.0f, e2 = 0.0f;
 #pragma unroll
         for (int i = 1; i < Q; i++) {
             const float t = s + g[i], z = t - s;
-            e += (s - (t - z)) + (g[i] - z);
+            const float d = (s - (t - z)) + (g[i] - z);
             s = t;
+            const float t2 = e + d, z2 = t2 - e;
+            e2 += (e - (t2 - z2)) + (d - z2);
+            e = t2;
         }
-        if (isfinite(s)) return (double)s + (double)e;
+        if (isfinite(s)) return (double)s + ((double)e + (double)e2);
         double dev = 0.0;  // diverged: the plain sum keeps infinities
         for (int i = 0; i < Q; i++) dev += (double)g[i];
         return dev;
