@@ -46,8 +46,7 @@ struct SlotDev {
     unsigned* rng;         // two-entry step counter for binary16 stochastic rounding
     int cpt;               // 32-cell row segments per stream-collide work item
     double* q;
-    double* q2;                 // second position buffer of the fused ring kernel (2D)
-    double* phi;
+    double* phi;                // nodal forces; second position buffer of the fused ring kernel
     int N, M;
     int* tri;
     int* csr_ptr;
@@ -407,7 +406,7 @@ k_b_interp(const SlotDev* __restrict__ slots, const int2* __restrict__ nodes, in
     if (t >= nnodes) return;
     const int2 nd = nodes[t];
     const SlotDev& sd = slots[nd.x];
-    const double* q = (D == 2 && sel) ? sd.q2 : sd.q;
+    const double* q = (D == 2 && sel) ? sd.phi : sd.q;
     R acc[3];
     interp_node<D, R>(sd.g, q, (const R*)sd.mom, nd.y, acc);
     for (int k = 0; k < D; k++) sd.q[D * nd.y + k] = q[D * nd.y + k] + (double)acc[k];
@@ -422,7 +421,7 @@ k_b_ring(const SlotDev* __restrict__ slots, const int2* __restrict__ rings, int 
 {
     const int2 it = rings[blockIdx.x];
     const SlotDev& sd = slots[it.x];
-    ring_warp<R, FIRST>(sd.g, sel ? sd.q2 : sd.q, sel ? sd.q : sd.q2, sd.N, it.y, sd.fp,
+    ring_warp<R, FIRST>(sd.g, sel ? sd.phi : sd.q, sel ? sd.q : sd.phi, sd.N, it.y, sd.fp,
                         (const R*)sd.mom, (R*)sd.F, sd.flags, sd.err);
 }
 
@@ -515,7 +514,7 @@ __global__ void k_b_classify(const SlotDev* __restrict__ slots, const int2* __re
     const SlotDev& sd = slots[it.x];
     if (!sd.two_tau) return;
     if (dim == 2)
-        classify_segment(sel ? sd.q2 : sd.q, sd.N, it.y, sd.g, sd.col_cnt, sd.col_z, sd.err);
+        classify_segment(sel ? sd.phi : sd.q, sd.N, it.y, sd.g, sd.col_cnt, sd.col_z, sd.err);
     else
         classify_face(sd.q, sd.tri, it.y, sd.g, sd.col_cnt, sd.col_z, sd.err);
 }
@@ -613,7 +612,7 @@ struct Arena {
 };
 
 struct Layout {
-    size_t pop[2], mom, F, flags, err, rng, q, q2, phi, tri, csr, epos, erec, eref, cols, colz, total;
+    size_t pop[2], mom, F, flags, err, rng, q, phi, tri, csr, epos, erec, eref, cols, colz, total;
 };
 
 Layout slot_layout(int Q, int dim, size_t elt, size_t relt, long long ncell, int rowlen, int N,
@@ -635,7 +634,6 @@ Layout slot_layout(int Q, int dim, size_t elt, size_t relt, long long ncell, int
     L.err = take(sizeof(int));
     L.rng = take(2 * sizeof(unsigned));
     L.q = take(sizeof(double) * (size_t)N * dim);
-    if (dim == 2 && elt != 2) L.q2 = take(sizeof(double) * (size_t)N * dim);
     L.phi = take(sizeof(double) * (size_t)N * dim);
     if (dim == 3) {
         L.tri = take(sizeof(int) * 3 * (size_t)M);
@@ -1372,7 +1370,6 @@ iblb_status iblb_batch_admit(iblb_batch b, const iblb_config* cfg, const double*
     d.scale = b->storage == IBLB_FP16_DEV ? std::ldexp(1.0f, sexp) : 1.0f;
     d.inv_scale = 1.0f / d.scale;
     d.q = (double*)(base + L.q);
-    d.q2 = (dim == 2 && b->elt != 2) ? (double*)(base + L.q2) : nullptr;
     d.phi = (double*)(base + L.phi);
     d.N = n_nodes;
     d.M = dim == 3 ? n_faces : n_nodes;

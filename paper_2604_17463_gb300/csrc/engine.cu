@@ -67,8 +67,8 @@ struct iblb_sim {
     // interface
     int N = 0, M = 0;
     double* q = nullptr;         // node positions
-    double* q2 = nullptr;        // 2D: second buffer of the fused ring kernel (swapped with q)
-    double* phi = nullptr;
+    double* phi = nullptr;       // nodal forces; the fused ring kernel, which keeps its forces in
+                                 // registers, moves the positions here and swaps the two
     int* tri = nullptr;
     int* csr_ptr = nullptr;
     int* entry_pos = nullptr;    // CSR position of each (face, corner) (3D)
@@ -303,7 +303,7 @@ void enqueue_band_cells(iblb_sim* h, cudaStream_t s)
 // after an even number of steps.
 void enqueue_ring_steps(iblb_sim* h, cudaStream_t s, int steps, bool last)
 {
-    double *q = h->q, *other = h->q2;
+    double *q = h->q, *other = h->phi;
     for (int k = 0; k < steps; k++) {
         launch_ring(h->storage, k == 0, q, other, h->N, h->fp, h->mom, h->F, h->flags, h->g, h->err, s);
         if (k > 0) std::swap(q, other);
@@ -678,7 +678,6 @@ void iblb_destroy(iblb_handle h)
     free_dev(h->obs_ws);
     h->read_ws.release();
     free_dev(h->q);
-    free_dev(h->q2);
     free_dev(h->phi);
     free_dev(h->tri);
     free_dev(h->csr_ptr);
@@ -748,7 +747,6 @@ iblb_status iblb_set_interface(iblb_handle h, const double* xyz, int n_nodes, co
     CK(h, cudaStreamSynchronize(h->stream));
     clear_graphs(h);
     free_dev(h->q);
-    free_dev(h->q2);
     free_dev(h->phi);
     free_dev(h->tri);
     free_dev(h->csr_ptr);
@@ -766,7 +764,6 @@ iblb_status iblb_set_interface(iblb_handle h, const double* xyz, int n_nodes, co
     if (n_nodes == 0) return IBLB_OK;
     const size_t qb = sizeof(double) * (size_t)n_nodes * dim;
     CK(h, cudaMalloc(&h->q, qb));
-    if (dim == 2 && h->storage != IBLB_FP16_DEV) CK(h, cudaMalloc(&h->q2, qb));
     CK(h, cudaMalloc(&h->phi, qb));
     CK(h, cudaMemcpyAsync(h->q, xyz, qb, cudaMemcpyHostToDevice, h->stream));
     if (h->det) {
@@ -831,7 +828,7 @@ iblb_status iblb_step(iblb_handle h, int n_steps)
         CK(h, cudaGraphLaunch(ge, h->stream));
         g_launches += graph_kernels(h, k, ring);
         h->cur ^= (k & 1);
-        if (ring && k % 2 == 0) std::swap(h->q, h->q2);
+        if (ring && k % 2 == 0) std::swap(h->q, h->phi);
         left -= k;
     }
     return IBLB_OK;
