@@ -707,7 +707,6 @@ struct iblb_batch_s {
     bool any_ext = false;     // an active slot has moving walls or a viscosity ratio
     double* d_partial = nullptr;
     double* d_obs = nullptr;
-    Workspace read_ws;            // FP64 fields of iblb_batch_read_fields
     double* d_obs_ws = nullptr;  // workspace of the observables, from the first call on
     int par = 0;
     bool dirty = true;
@@ -1280,7 +1279,6 @@ void iblb_batch_destroy(iblb_batch b)
     cudaFree(b->d_partial);
     cudaFree(b->d_obs);
     cudaFree(b->d_obs_ws);
-    b->read_ws.release();
     for (cudaStream_t st : {b->cap[0], b->cap[1], b->low[0], b->low[1]})
         if (st) cudaStreamDestroy(st);
     for (cudaEvent_t ev : {b->ev_fork, b->ev_join, b->ev_ib, b->ev_sc})
@@ -1653,8 +1651,8 @@ iblb_status iblb_batch_read_fields(iblb_batch b, int slot, double* rho, double* 
     const SlotDev& d = sl.dev;
     const long long nc = d.g.ncell;
     if (rho || u) {
-        BCK(b, b->read_ws.need(sizeof(double) * (size_t)(1 + b->dim) * nc));
-        double* tmp = (double*)b->read_ws.p;
+        double* tmp = nullptr;
+        BCK(b, cudaMalloc(&tmp, sizeof(double) * (size_t)(1 + b->dim) * nc));
         launch_unpack_moments(b->storage, d.g, d.mom, tmp, tmp + nc, b->stream);
         b->launches++;
         add_launches(1);
@@ -1665,7 +1663,7 @@ iblb_status iblb_batch_read_fields(iblb_batch b, int slot, double* rho, double* 
             e = cudaMemcpyAsync(u, tmp + nc, sizeof(double) * b->dim * nc, cudaMemcpyDeviceToHost,
                                 b->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-        b->read_ws.trim();
+        cudaFree(tmp);
         if (e != cudaSuccess) return bfail(b, IBLB_ECUDA, cudaGetErrorString(e));
     }
     if (xyz)

@@ -353,36 +353,6 @@ void launch_classify(int dim, const double* q, int N, const int* tri, int M, con
 void launch_inside_mask(const GridParams& g, const int* cnt, const double* cz,
                         unsigned char* mask, cudaStream_t s);
 
-// Device workspace that an object keeps between calls, grown to the largest
-// request; one above KEEP_BYTES is given back by trim() at the end of the call.
-// Reading 64 small batch slots took 7.5 ms with an allocation per read, so 5.0;
-// 8 slots of up to 192 x 192 x 96 120 ms, so 72 to 100; 2048 x 512 0.37 ms, so
-// 0.20.
-struct Workspace {
-    static constexpr size_t KEEP_BYTES = (size_t)512 << 20;
-    void* p = nullptr;
-    size_t bytes = 0;
-    cudaError_t need(size_t n)
-    {
-        if (n <= bytes) return cudaSuccess;
-        release();
-        const cudaError_t e = cudaMalloc(&p, n);
-        if (e == cudaSuccess) bytes = n;
-        else p = nullptr;
-        return e;
-    }
-    void trim()
-    {
-        if (bytes > KEEP_BYTES) release();
-    }
-    void release()
-    {
-        if (p) cudaFree(p);
-        p = nullptr;
-        bytes = 0;
-    }
-};
-
 // Kernel-launch accounting shared by the engines (iblb_kernel_launch_count).
 void add_launches(long long n);
 

@@ -62,7 +62,6 @@ struct iblb_sim {
     double* partial = nullptr;
     int npartial = 0;
     double* obs = nullptr;     // 12 doubles
-    Workspace read_ws;         // FP64 fields of iblb_read_fields
     double* obs_ws = nullptr;  // workspace of observables and deformation, from the first call on
     // interface
     int N = 0, M = 0;
@@ -676,7 +675,6 @@ void iblb_destroy(iblb_handle h)
     free_dev(h->partial);
     free_dev(h->obs);
     free_dev(h->obs_ws);
-    h->read_ws.release();
     free_dev(h->q);
     free_dev(h->phi);
     free_dev(h->tri);
@@ -856,8 +854,8 @@ iblb_status iblb_read_fields(iblb_handle h, double* rho, double* u, double* xyz)
     if (!h) return IBLB_EINVAL;
     const long long nc = h->g.ncell;
     if (rho || u) {
-        CK(h, h->read_ws.need(sizeof(double) * (size_t)(1 + h->dim) * nc));
-        double* tmp = (double*)h->read_ws.p;
+        double* tmp = nullptr;
+        CK(h, cudaMalloc(&tmp, sizeof(double) * (size_t)(1 + h->dim) * nc));
         launch_unpack_moments(h->storage, h->g, h->mom, tmp, tmp + nc, h->stream);
         g_launches++;
         cudaError_t e = cudaGetLastError();
@@ -867,7 +865,7 @@ iblb_status iblb_read_fields(iblb_handle h, double* rho, double* u, double* xyz)
             e = cudaMemcpyAsync(u, tmp + nc, sizeof(double) * h->dim * nc, cudaMemcpyDeviceToHost,
                                 h->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-        h->read_ws.trim();
+        cudaFree(tmp);
         if (e != cudaSuccess) return cuda_fail(h, e, "read_fields");
     }
     if (xyz && h->N > 0)
