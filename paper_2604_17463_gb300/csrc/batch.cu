@@ -707,7 +707,6 @@ struct iblb_batch_s {
     bool any_ext = false;     // an active slot has moving walls or a viscosity ratio
     double* d_partial = nullptr;
     double* d_obs = nullptr;
-    double* d_obs_ws = nullptr;  // workspace of the observables, from the first call on
     int par = 0;
     bool dirty = true;
     int sm_count = 0;
@@ -1235,7 +1234,7 @@ iblb_status iblb_batch_create(int lattice, int storage, size_t hbm_budget_bytes,
     if (e == cudaSuccess) e = cudaMalloc(&b->arena_ptr, budget);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_slots, sizeof(SlotDev) * max_slots);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_partial, sizeof(double) * 1024);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_obs, sizeof(double) * 12);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_obs, sizeof(double) * (12 + OBS_WS * OBS_GRID));
     int lo = 0, hi = 0;
     if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
     for (int k = 0; k < 2; k++) {
@@ -1278,7 +1277,6 @@ void iblb_batch_destroy(iblb_batch b)
     cudaFree(b->detb.wts);
     cudaFree(b->d_partial);
     cudaFree(b->d_obs);
-    cudaFree(b->d_obs_ws);
     for (cudaStream_t st : {b->cap[0], b->cap[1], b->low[0], b->low[1]})
         if (st) cudaStreamDestroy(st);
     for (cudaEvent_t ev : {b->ev_fork, b->ev_join, b->ev_ib, b->ev_sc})
@@ -1620,10 +1618,10 @@ iblb_status iblb_batch_observables(iblb_batch b, int slot, iblb_obs* out)
         return IBLB_EINVAL;
     Slot& sl = b->slots[slot];
     const SlotDev& d = sl.dev;
-    if (!b->d_obs_ws) BCK(b, cudaMalloc(&b->d_obs_ws, sizeof(double) * OBS_WS));
     launch_mass_partials(b->Q, b->storage, d.f[sl.buf], d.g, d.inv_scale, b->d_partial, b->stream);
     launch_observables(b->dim, d.q, d.N, b->dim == 3 ? d.tri : nullptr, d.M, b->d_partial,
-                       mass_partial_blocks(d.g), sl.cfg.xi, 0.5, b->d_obs, b->d_obs_ws, b->stream);
+                       mass_partial_blocks(d.g), sl.cfg.xi, 0.5, b->d_obs, b->d_obs + 12, OBS_GRID,
+                       b->stream);
     b->launches += 1 + OBS_KERNELS;
     add_launches(1 + OBS_KERNELS);
     BCK(b, cudaGetLastError());

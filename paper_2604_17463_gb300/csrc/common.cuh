@@ -315,22 +315,23 @@ void launch_elastic_reference(int dim, const double* q, int N, int M, const int*
                               cudaStream_t s);
 
 // Observables (deterministic; OBS_KERNELS kernels).  out: 12 doubles, layout of
-// iblb_obs; ws: OBS_WS doubles of workspace.
+// iblb_obs; ws: workspace of OBS_WS doubles for each of `blocks` blocks (1 ..
+// OBS_GRID), which is the most that a kernel is launched with.
 constexpr int OBS_GRID = 64;
-constexpr int OBS_WS = 30 * OBS_GRID;
+constexpr int OBS_WS = 30;
 constexpr int OBS_KERNELS = 4;
 void launch_observables(int dim, const double* q, int N, const int* tri, int M,
                         const double* mass_partial, int n_partial, double xi, double wall_plane,
-                        double* out, double* ws, cudaStream_t s);
+                        double* out, double* ws, int blocks, cudaStream_t s);
 
 // f = f_eq(rho, u) in storage form (deviation from w, scaled); rho may be null (1).
 void launch_set_equilibrium(int Q, int storage, int dim, const double* rho, const double* u,
                             void* dst, long long ncell, float scale, cudaStream_t s);
 // Deformation index of the interface in the shear plane: out[5] =
-// {D, r1, r3, inclination (deg), enclosed area / volume}; ws: OBS_WS doubles.
+// {D, r1, r3, inclination (deg), enclosed area / volume}; ws, blocks: as above.
 constexpr int DEFORMATION_KERNELS = 3;
 void launch_deformation(int dim, const double* q, int N, const int* tri, int M, double* out,
-                        double* ws, cudaStream_t s);
+                        double* ws, int blocks, cudaStream_t s);
 
 // Inside / outside test of the cell at wall-axis coordinate a in column col:
 // an odd number of interface crossings below it.

@@ -61,8 +61,7 @@ struct iblb_sim {
     int* err = nullptr;
     double* partial = nullptr;
     int npartial = 0;
-    double* obs = nullptr;     // 12 doubles
-    double* obs_ws = nullptr;  // workspace of observables and deformation, from the first call on
+    double* obs = nullptr;     // 12 doubles, then the workspace of one block (obs_workspace)
     // interface
     int N = 0, M = 0;
     double* q = nullptr;         // node positions
@@ -352,6 +351,16 @@ void enqueue_step_overlapped(iblb_sim* h, cudaStream_t a, cudaStream_t b, bool w
     h->cur ^= 1;
 }
 
+// Workspace of the observables and the deformation: the band list, which holds
+// nothing between steps; on a lattice with too few segments one block's at the
+// end of `obs`.  The calls allocate nothing.
+double* obs_workspace(iblb_sim* h, int* blocks)
+{
+    const long long fit = (long long)(sizeof(int) * 4 * h->nflags / (sizeof(double) * OBS_WS));
+    *blocks = (int)std::max(1LL, std::min((long long)OBS_GRID, fit));
+    return fit >= 1 ? (double*)h->band_list : h->obs + 12;
+}
+
 iblb_status get_graph(iblb_sim* h, int steps, bool last, bool ring, cudaGraphExec_t* out)
 {
     auto key = std::make_tuple(h->cur, steps, (last ? 1 : 0) + (ring ? 2 : 0), h->q);
@@ -575,7 +584,7 @@ iblb_status iblb_create(const iblb_config* cfg, void* cuda_stream, iblb_handle* 
     h->npartial = mass_partial_blocks(g);
     if ((e = cudaMalloc(&h->partial, sizeof(double) * h->npartial)) != cudaSuccess)
         return bail(e, "partial");
-    if ((e = cudaMalloc(&h->obs, sizeof(double) * 12)) != cudaSuccess) return bail(e, "obs");
+    if ((e = cudaMalloc(&h->obs, sizeof(double) * (12 + OBS_WS))) != cudaSuccess) return bail(e, "obs");
     if ((e = cudaMalloc(&h->defo, sizeof(double) * 8)) != cudaSuccess) return bail(e, "obs");
     if ((e = cudaMalloc(&h->rng, sizeof(unsigned) * 2)) != cudaSuccess) return bail(e, "obs");
     cudaMemsetAsync(h->rng, 0, sizeof(unsigned) * 2, h->stream);
@@ -674,7 +683,6 @@ void iblb_destroy(iblb_handle h)
     free_dev(h->err);
     free_dev(h->partial);
     free_dev(h->obs);
-    free_dev(h->obs_ws);
     free_dev(h->q);
     free_dev(h->phi);
     free_dev(h->tri);
@@ -914,11 +922,12 @@ iblb_status iblb_get_populations(iblb_handle h, double* f)
 iblb_status iblb_observables(iblb_handle h, iblb_obs* out)
 {
     if (!h || !out) return IBLB_EINVAL;
-    if (!h->obs_ws) CK(h, cudaMalloc(&h->obs_ws, sizeof(double) * OBS_WS));
+    int blocks;
+    double* ws = obs_workspace(h, &blocks);
     launch_mass_partials(h->Q, h->storage, h->f[h->cur], h->g, h->sp.inv_scale, h->partial,
                          h->stream);
     launch_observables(h->dim, h->q, h->N, h->tri, h->M, h->partial, h->npartial, h->cfg.xi, 0.5,
-                       h->obs, h->obs_ws, h->stream);
+                       h->obs, ws, blocks, h->stream);
     g_launches += 1 + OBS_KERNELS;
     CK(h, cudaGetLastError());
     double v[12];
@@ -1050,8 +1059,9 @@ iblb_status iblb_deformation(iblb_handle h, double* out)
     if (!h || !out) return IBLB_EINVAL;
     if (h->N < 3 || (h->dim == 3 && h->M < 4))
         return fail(h, IBLB_EINVAL, "deformation needs a closed interface");
-    if (!h->obs_ws) CK(h, cudaMalloc(&h->obs_ws, sizeof(double) * OBS_WS));
-    launch_deformation(h->dim, h->q, h->N, h->tri, h->M, h->defo, h->obs_ws, h->stream);
+    int blocks;
+    double* ws = obs_workspace(h, &blocks);
+    launch_deformation(h->dim, h->q, h->N, h->tri, h->M, h->defo, ws, blocks, h->stream);
     g_launches += DEFORMATION_KERNELS;
     CK(h, cudaGetLastError());
     CK(h, cudaMemcpyAsync(out, h->defo, sizeof(double) * 5, cudaMemcpyDeviceToHost, h->stream));

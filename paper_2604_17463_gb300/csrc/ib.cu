@@ -318,7 +318,7 @@ struct ObsArgs {
     int n_partial;
     double xi, wp;
     double* out;           // 12 results
-    double *p1, *p2, *p3;  // partial sums [OBS_GRID][...]
+    double *p1, *p2, *p3;  // partial sums [block][...]
 };
 
 // Sums over the blocks of column k of a partial array, by the first warp
@@ -609,14 +609,14 @@ __global__ void __launch_bounds__(32) k_def_last(int dim, const double* __restri
 }
 
 void launch_deformation(int dim, const double* q, int N, const int* tri, int M, double* out,
-                        double* ws, cudaStream_t s)
+                        double* ws, int blocks, cudaStream_t s)
 {
     const int n = dim == 2 ? N : (M > N ? M : N);
     int grid = (n + OBS_THREADS - 1) / OBS_THREADS;
-    grid = grid < 1 ? 1 : (grid > OBS_GRID ? OBS_GRID : grid);
+    grid = grid < 1 ? 1 : (grid > blocks ? blocks : grid);
     double* mean_part = ws;
-    double* part = mean_part + 3 * OBS_GRID;
-    static_assert(9 * OBS_GRID <= OBS_WS, "deformation workspace");
+    double* part = mean_part + 3 * grid;
+    static_assert(9 <= OBS_WS, "deformation workspace");
     k_def_mean<<<grid, OBS_THREADS, 0, s>>>(dim, q, N, mean_part);
     k_def_moments<<<grid, OBS_THREADS, 0, s>>>(dim, q, N, tri, M, mean_part, part);
     k_def_last<<<1, 32, 0, s>>>(dim, part, grid, out);
@@ -624,15 +624,15 @@ void launch_deformation(int dim, const double* q, int N, const int* tri, int M, 
 
 void launch_observables(int dim, const double* q, int N, const int* tri, int M,
                         const double* mass_partial, int n_partial, double xi, double wall_plane,
-                        double* out, double* ws, cudaStream_t s)
+                        double* out, double* ws, int blocks, cudaStream_t s)
 {
     ObsArgs a{dim, q, N, tri, M, mass_partial, n_partial, xi, wall_plane, out, nullptr, nullptr, nullptr};
-    a.p1 = ws;
-    a.p2 = a.p1 + OBS_P1 * OBS_GRID;
-    a.p3 = a.p2 + OBS_P2 * OBS_GRID;
-    static_assert((OBS_P1 + OBS_P2 + OBS_P3) * OBS_GRID <= OBS_WS, "observables workspace");
     int grid = ((N > n_partial ? N : n_partial) + OBS_THREADS - 1) / OBS_THREADS;
-    grid = grid < 1 ? 1 : (grid > OBS_GRID ? OBS_GRID : grid);
+    grid = grid < 1 ? 1 : (grid > blocks ? blocks : grid);
+    a.p1 = ws;
+    a.p2 = a.p1 + OBS_P1 * grid;
+    a.p3 = a.p2 + OBS_P2 * grid;
+    static_assert(OBS_P1 + OBS_P2 + OBS_P3 <= OBS_WS, "observables workspace");
     k_obs_sums<<<grid, OBS_THREADS, 0, s>>>(a);
     k_obs_fit<<<grid, OBS_THREADS, 0, s>>>(a);
     k_obs_film<<<grid, OBS_THREADS, 0, s>>>(a);
