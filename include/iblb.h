@@ -258,7 +258,7 @@ iblb_status iblb_step_profiled(iblb_handle h, int n_steps, double* kernel_ms);
 /* Launch shape of the stream-collide kernel.  Results do not depend on the
  * sizes of a variant; two variants round some sums differently (FP64, FP32: in
  * the last bits; binary16: another realisation of the stochastic rounding),
- * but for D2Q9 with binary16 storage, where variants 0 and 1 give the same bits.
+ * but in binary16 storage variants 0 and 1 give the same bits.
  *   variant 0: the plain kernel, one cell per thread, block_x threads per
  *              block along x (64, 128 or 256), evict-first stores of the new
  *              populations when streaming_stores != 0;
@@ -311,7 +311,9 @@ typedef struct {
                                      updates the cells of the flagged band
                                      segments again, from the same sources,
                                      with their force density (the same
-                                     arithmetic as one pass).  Not used by
+                                     arithmetic as one pass; D3Q19 binary16
+                                     on widths that variant 1 takes: but for
+                                     the rounding of f_0).  Not used by
                                      iblb_step_profiled.  Not changed by
                                      iblb_autotune. */
 } iblb_tuning;

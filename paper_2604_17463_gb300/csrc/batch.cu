@@ -398,7 +398,7 @@ k_b_spread(const SlotDev* __restrict__ slots, const int2* __restrict__ nodes, in
 // One thread per (slot, node): interpolate and advect (interp_node).  The
 // positions are read from the second buffer when `sel` is set, and written to
 // the first.
-template <int D, typename R>
+template <int D, typename R, bool KEEP = keep_weights<D, R>>
 __global__ void __launch_bounds__(128)
 k_b_interp(const SlotDev* __restrict__ slots, const int2* __restrict__ nodes, int nnodes, int sel)
 {
@@ -408,7 +408,7 @@ k_b_interp(const SlotDev* __restrict__ slots, const int2* __restrict__ nodes, in
     const SlotDev& sd = slots[nd.x];
     const double* q = (D == 2 && sel) ? sd.phi : sd.q;
     R acc[3];
-    interp_node<D, R>(sd.g, q, (const R*)sd.mom, nd.y, acc);
+    interp_node<D, R, KEEP>(sd.g, q, (const R*)sd.mom, nd.y, acc);
     for (int k = 0; k < D; k++) sd.q[D * nd.y + k] = q[D * nd.y + k] + (double)acc[k];
 }
 
@@ -520,7 +520,8 @@ __global__ void k_b_classify(const SlotDev* __restrict__ slots, const int2* __re
 }
 
 static void launch_b_ib(int dim, int storage, int phase, const SlotDev* slots, const int2* nodes,
-                        int nnodes, const int2* faces, int nfaces, cudaStream_t s, int sel = 0)
+                        int nnodes, const int2* faces, int nfaces, cudaStream_t s, int sel = 0,
+                        bool ordered = false)
 {
     const int wb = 128;
     const int node_grid = (nnodes + wb - 1) / wb;  // one thread per (slot, node)
@@ -547,6 +548,7 @@ static void launch_b_ib(int dim, int storage, int phase, const SlotDev* slots, c
             else k_b_interp<3, double><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes, sel);
         } else {
             if (dim == 2) k_b_interp<2, float><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes, sel);
+            else if (keep_weights_3d(storage, ordered)) k_b_interp<3, float, true><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes, sel);
             else k_b_interp<3, float><<<node_grid, wb, 0, s>>>(slots, nodes, nnodes, sel);
         }
     }
@@ -1009,7 +1011,7 @@ void enqueue_sc(iblb_batch_s* b, cudaStream_t s, const Part& p, int par, bool wr
 
 void enqueue_interp(iblb_batch_s* b, cudaStream_t s, const Part& p, int sel = 0)
 {
-    launch_b_ib(b->dim, b->storage, 2, b->d_slots, b->d_nodes + p.n0, p.n1 - p.n0, nullptr, 0, s, sel);
+    launch_b_ib(b->dim, b->storage, 2, b->d_slots, b->d_nodes + p.n0, p.n1 - p.n0, nullptr, 0, s, sel, b->det);
 }
 
 // `steps` batched steps of one part from parity `par`, all phases over its
@@ -1520,8 +1522,7 @@ iblb_status batch_run(iblb_batch_s* b, int max_steps, int* n_completed, double* 
                             b->ntiles, b->par, grid, b->stream);
                 cudaEventRecord(ev[3], b->stream);
                 if (b->nnodes > 0)
-                    launch_b_ib(b->dim, b->storage, 2, b->d_slots, b->d_nodes, b->nnodes,
-                                b->d_faces, b->nfaces, b->stream);
+                    enqueue_interp(b, b->stream, all);
                 cudaEventRecord(ev[4], b->stream);
                 b->par ^= 1;
                 b->launches += kernels_per_step(b);

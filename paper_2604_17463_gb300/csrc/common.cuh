@@ -83,7 +83,7 @@ struct StreamParams {
     float omega_f;         // the same in FP32 (no per-thread conversion on the FP32 paths)
     float body_f[3];
     int has_body;          // any component of the body force is not zero
-    int rest_fused;        // D2Q9 binary16: see cell_update_h9
+    int rest_fused;        // binary16: see cell_update_h
     // viscosity ratio: cells outside the interface relax with omega_out
     int two_tau;
     double omega_out;
@@ -267,9 +267,10 @@ void launch_mesh_spread(int storage, const double* q, int N, int M, const int* t
                         const int* csr_ptr, const int* entry_pos, double* entry_rec,
                         const ForceParams& fp, void* F, uint8_t* flags, uint8_t* fine,
                         const GridParams& g, int* err, cudaStream_t s);
-// qdot [N][dim] = sum u Delta; if advect, q += qdot.
+// qdot [N][dim] = sum u Delta; if advect, q += qdot.  ordered: the run spreads
+// in order.
 void launch_interp(int storage, int dim, double* q, const void* moments, int N, double* qdot,
-                   bool advect, const GridParams& g, cudaStream_t s);
+                   bool advect, bool ordered, const GridParams& g, cudaStream_t s);
 
 // Spatial groups of 3D interface nodes (ib_groups.cu): nodes of one
 // GROUP_TILE^3 tile of the lattice, at most GROUP_NODES per group; the
@@ -306,7 +307,7 @@ void launch_spread_grouped(int storage, const double* q, const double* phi, cons
                            void* F, uint8_t* flags, const GridParams& g, int sm_count,
                            cudaStream_t s);
 void launch_interp_grouped(int storage, double* q, const void* moments, const NodeGroups& ng,
-                           double* qdot, bool advect, const GridParams& g, int sm_count,
+                           double* qdot, bool advect, bool ordered, const GridParams& g, int sm_count,
                            cudaStream_t s);
 
 // Elastic reference of the interface at its current positions (see

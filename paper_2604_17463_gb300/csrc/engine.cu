@@ -211,9 +211,10 @@ void enqueue_spread(iblb_sim* h, cudaStream_t s, bool band_pass = false)
 void enqueue_interp(iblb_sim* h, cudaStream_t s, const void* moments, double* qdot, bool advect)
 {
     if (use_groups(h))
-        launch_interp_grouped(h->storage, h->q, moments, h->grp, qdot, advect, h->g, h->sm_count, s);
+        launch_interp_grouped(h->storage, h->q, moments, h->grp, qdot, advect, h->det, h->g,
+                              h->sm_count, s);
     else
-        launch_interp(h->storage, h->dim, h->q, moments, h->N, qdot, advect, h->g, s);
+        launch_interp(h->storage, h->dim, h->q, moments, h->N, qdot, advect, h->det, h->g, s);
 }
 
 // A1 - A3: nodal forces and spread.
@@ -309,7 +310,7 @@ void enqueue_ring_steps(iblb_sim* h, cudaStream_t s, int steps, bool last)
         launch_sc(h, s, last && k == steps - 1);
         h->cur ^= 1;
     }
-    launch_interp(h->storage, 2, q, h->mom, h->N, nullptr, true, h->g, s);
+    launch_interp(h->storage, 2, q, h->mom, h->N, nullptr, true, false, h->g, s);
 }
 
 // One overlapped time step under graph capture.  Stream b runs the bulk
@@ -658,7 +659,7 @@ iblb_status iblb_create(const iblb_config* cfg, void* cuda_stream, iblb_handle* 
     if ((e = prepare_stream_collide_pipe(h->smem)) != cudaSuccess) return bail(e, "pipe attributes");
     h->sm_count = sms;
     // walls that move and a viscosity ratio always run the plain kernel
-    if (h->Q == 9 && h->storage == IBLB_FP16_DEV && !h->moving && !h->two_tau) {
+    if (h->storage == IBLB_FP16_DEV && !h->moving && !h->two_tau) {
         const Tuning t;
         PipeShape ps{};
         sp.rest_fused = pipe_shape(h->Q, h->storage, g, sms, h->smem, t.rows_per_tile, t.ctas_per_sm,

@@ -189,7 +189,7 @@ void launch_mesh_spread(int storage, const double* q, int N, int M, const int* t
 // One thread per node (interp_node in ib_core.cuh): 16 velocity reads in
 // flight per thread; on the 59 292-node mesh 16 us per step against 35 us
 // for one warp per node with two reads per lane and a shuffle reduction.
-template <int D, typename R>
+template <int D, typename R, bool KEEP = keep_weights<D, R>>
 __global__ void __launch_bounds__(128)
 k_interp_t(double* __restrict__ q, const R* __restrict__ mom, int N, double* __restrict__ qdot,
            int advect, GridParams g)
@@ -197,7 +197,7 @@ k_interp_t(double* __restrict__ q, const R* __restrict__ mom, int N, double* __r
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= N) return;
     R acc[3];
-    interp_node<D, R>(g, q, mom, j, acc);
+    interp_node<D, R, KEEP>(g, q, mom, j, acc);
     for (int k = 0; k < D; k++) {
         if (qdot) qdot[D * j + k] = (double)acc[k];
         if (advect) q[D * j + k] += (double)acc[k];
@@ -205,7 +205,7 @@ k_interp_t(double* __restrict__ q, const R* __restrict__ mom, int N, double* __r
 }
 
 void launch_interp(int storage, int dim, double* q, const void* moments, int N, double* qdot,
-                   bool advect, const GridParams& g, cudaStream_t s)
+                   bool advect, bool ordered, const GridParams& g, cudaStream_t s)
 {
     if (N <= 0) return;
     const int b = node_block(storage, dim, N), grid = (N + b - 1) / b;
@@ -214,6 +214,7 @@ void launch_interp(int storage, int dim, double* q, const void* moments, int N, 
         else k_interp_t<3, double><<<grid, b, 0, s>>>(q, (const double*)moments, N, qdot, advect, g);
     } else {
         if (dim == 2) k_interp_t<2, float><<<grid, b, 0, s>>>(q, (const float*)moments, N, qdot, advect, g);
+        else if (keep_weights_3d(storage, ordered)) k_interp_t<3, float, true><<<grid, b, 0, s>>>(q, (const float*)moments, N, qdot, advect, g);
         else k_interp_t<3, float><<<grid, b, 0, s>>>(q, (const float*)moments, N, qdot, advect, g);
     }
 }

@@ -49,14 +49,22 @@ __device__ __forceinline__ float delta4f(float r)
 // branches of the kernel diverging in the warp, and with one-warp blocks, the
 // step of the FP64 128 x 64 ring (213 nodes) went from 34.7 to 25.4 us.
 //
-// 2D interfaces in FP32 keep one root per weight (cheap there): the ring's
-// forces then round as they always have, and a binary16 run, whose stochastic
-// rounding turns any change of a last bit into another trajectory, keeps its
-// own.
+// KEEP: one root per weight.  A binary16 run, whose stochastic rounding turns
+// any change of a last bit into another trajectory, keeps its weights to the bit
+// where it is a function of its inputs: 2D interfaces in FP32 (cheap there), and
+// 3D binary16 runs with the ordered spread.  In the other 3D runs the order of
+// the additions varies more than the weights do, and one root per weight would
+// cost the binary16 256 x 256 x 128 drop (40 962 nodes) 35.2 -> 39.1 ms per pass
+// of 200 steps, the FP32 101 x 101 x 77 one 15.6 -> 16.2 ms of 300.
 template <int D, typename R>
+constexpr bool keep_weights = D == 2 && sizeof(R) == 4;
+// 3D: whether a run keeps them.
+constexpr bool keep_weights_3d(int storage, bool ordered) { return storage == ST_FP16 && ordered; }
+
+template <typename R, bool KEEP>
 __device__ __forceinline__ void delta4_weights(R fr, R (&w)[4])
 {
-    if constexpr (D == 2 && sizeof(R) == 4) {
+    if constexpr (KEEP) {
 #pragma unroll
         for (int o = 0; o < 4; o++) w[o] = delta4f(fr + (float)(1 - o));
         return;
@@ -74,7 +82,7 @@ __device__ __forceinline__ void delta4_weights(R fr, R (&w)[4])
 // the node coordinate, once per axis) and lattice indices (wrapped on periodic axes, -1 on
 // a solid layer or outside the lattice along the wall axis).  Returns false
 // for a diverged node (it touches nothing).
-template <int D, typename R>
+template <int D, typename R, bool KEEP = keep_weights<D, R>>
 __device__ __forceinline__ bool node_lines(const GridParams& g, const double* __restrict__ q,
                                            int node, R (&w)[3][4], int (&ix)[3][4])
 {
@@ -111,7 +119,7 @@ __device__ __forceinline__ bool node_lines(const GridParams& g, const double* __
             }
             continue;
         }
-        delta4_weights<D, R>(fr, w[k]);
+        delta4_weights<R, KEEP>(fr, w[k]);
         int at = base % ext;
         at = at < 0 ? at + ext : at;
 #pragma unroll
@@ -208,14 +216,14 @@ __device__ __forceinline__ void spread_node(const GridParams& g, const double* _
 // Interpolated velocity at node j by one thread: the 16 / 64 velocity reads
 // of its stencil, 16 issued at a time (one 4 x 4 plane of points) before any
 // is used.
-template <int D, typename R>
+template <int D, typename R, bool KEEP = keep_weights<D, R>>
 __device__ __forceinline__ void interp_node(const GridParams& g, const double* __restrict__ q,
                                             const R* __restrict__ mom, int j, R (&acc)[3])
 {
     R w[3][4];
     int ix[3][4];
     acc[0] = acc[1] = acc[2] = R(0);
-    if (!node_lines<D, R>(g, q, j, w, ix)) return;
+    if (!node_lines<D, R, KEEP>(g, q, j, w, ix)) return;
     const int n2 = (D == 3) ? 4 : 1;
     for (int o2 = 0; o2 < n2; o2++) {
         const int i2 = ix[2][o2];

@@ -221,14 +221,14 @@ __device__ __forceinline__ long long box_cell(const GridParams& g, const GroupBo
 
 // 1D weights of node j along each axis (as node_lines: FP64 floor /
 // fraction split, weights in R).
-template <typename R>
+template <typename R, bool KEEP = false>
 __device__ __forceinline__ void node_weights3(const double* __restrict__ q, int j, R (&w)[3][4])
 {
 #pragma unroll
     for (int k = 0; k < 3; k++) {
         const double qk = q[3 * j + k];
         const double fl = floor(qk);
-        delta4_weights<3, R>((R)(qk - fl), w[k]);
+        delta4_weights<R, KEEP>((R)(qk - fl), w[k]);
     }
 }
 
@@ -351,7 +351,7 @@ k_spread_grouped(const double* __restrict__ q, const double* __restrict__ phi,
 // into shared memory (float4 (drho, ux, uy, uz) per cell in FP32, as the
 // moments are stored; three FP64 arrays otherwise), four cells per thread in
 // flight, then each thread sums its node's 64 stencil points from there.
-template <typename R>
+template <typename R, bool KEEP>
 __global__ void __launch_bounds__(GROUP_NODES)
 k_interp_grouped(double* __restrict__ q, const R* __restrict__ mom, NodeGroups ng,
                  double* __restrict__ qdot, int advect, GridParams g)
@@ -373,7 +373,7 @@ k_interp_grouped(double* __restrict__ q, const R* __restrict__ mom, NodeGroups n
         const bool has = d[0] != INT_MIN;
         R acc[3] = {R(0), R(0), R(0)};
         if (bx.vol == INT_MAX) {
-            if (has) interp_node<3, R>(g, q, mom, j, acc);
+            if (has) interp_node<3, R, KEEP>(g, q, mom, j, acc);
         } else {
             constexpr int U = 4;
             for (int c0 = threadIdx.x; c0 < bx.vol; c0 += U * GROUP_NODES) {
@@ -407,7 +407,7 @@ k_interp_grouped(double* __restrict__ q, const R* __restrict__ mom, NodeGroups n
             __syncthreads();
             if (has) {
                 R w[3][4];
-                node_weights3<R>(q, j, w);
+                node_weights3<R, KEEP>(q, j, w);
                 const int ox = d[0] - bx.m[0], oy = d[1] - bx.m[1], oz = d[2] - bx.m[2];
                 for (int o2 = 0; o2 < 4; o2++) {
 #pragma unroll
@@ -467,15 +467,18 @@ void launch_spread_grouped(int storage, const double* q, const double* phi, cons
 }
 
 void launch_interp_grouped(int storage, double* q, const void* moments, const NodeGroups& ng,
-                           double* qdot, bool advect, const GridParams& g, int sm_count,
+                           double* qdot, bool advect, bool ordered, const GridParams& g, int sm_count,
                            cudaStream_t s)
 {
     const int grid = grouped_grid(ng, sm_count);
     if (storage == ST_FP64)
-        k_interp_grouped<double><<<grid, GROUP_NODES, 0, s>>>(q, (const double*)moments, ng, qdot,
+        k_interp_grouped<double, false><<<grid, GROUP_NODES, 0, s>>>(q, (const double*)moments, ng, qdot,
                                                               advect ? 1 : 0, g);
+    else if (keep_weights_3d(storage, ordered))
+        k_interp_grouped<float, true><<<grid, GROUP_NODES, 0, s>>>(q, (const float*)moments, ng, qdot,
+                                                             advect ? 1 : 0, g);
     else
-        k_interp_grouped<float><<<grid, GROUP_NODES, 0, s>>>(q, (const float*)moments, ng, qdot,
+        k_interp_grouped<float, false><<<grid, GROUP_NODES, 0, s>>>(q, (const float*)moments, ng, qdot,
                                                              advect ? 1 : 0, g);
 }
 

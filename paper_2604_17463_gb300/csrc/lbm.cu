@@ -167,14 +167,14 @@ __device__ __forceinline__ void sc_cell(const typename StorageT<ST>::S* __restri
     const bool force = band || p.has_body;  // uniform in the warp
     if constexpr (D == 2) {
         if constexpr (ST == ST_FP16) {
-            mo = cell_update_h9<!BULK>(g, p.rest_fused, om, Fx, Fy, p.inv_scale, p.scale);
+            mo = cell_update_h<9, !BULK>(g, p.rest_fused, om, Fx, Fy, 0.0f, p.inv_scale, p.scale);
             store_cell32<Q, ST, CS>(fout, nc, c32, g, 1.0f, sr_seed(step, cell));
         } else {
             mo = cell_update<Q, R, FM>(g, force, om, Fx, Fy, Fz);
             store_cell32<Q, ST, CS>(fout, nc, c32, g, p.scale, 0u);
         }
     } else if constexpr (ST == ST_FP16) {
-        mo = cell_update<Q, R, FM>(g, force, om, Fx, Fy, Fz, (R)p.inv_scale, (R)p.scale);
+        mo = cell_update_h<19, !BULK>(g, p.rest_fused, om, Fx, Fy, Fz, p.inv_scale, p.scale);
         store_cell<Q, ST, CS>(fout, nc, cell, g, 1.0f, sr_seed(step, cell));
     } else {
         mo = cell_update<Q, R, FM>(g, force, om, Fx, Fy, Fz);
@@ -420,10 +420,11 @@ void launch_band_list(const uint8_t* flags, const uint8_t* fine, const GridParam
 
 template <int Q, int ST>
 static void launch_band_t(const void* fin, void* fout, void* mom, void* F, uint8_t* flags,
-                          uint8_t* fine, const int* list, const int* count, const StreamParams& p,
+                          uint8_t* fine, const int* list, const int* count, StreamParams p,
                           int sm_count, cudaStream_t s)
 {
     using T = StorageT<ST>;
+    if (Q == 19) p.rest_fused = 0;  // binary16: the band cells of 3D lattices never fuse it
     auto* a = (const typename T::S*)fin;
     auto* b = (typename T::S*)fout;
     auto* m = (typename T::R*)mom;

@@ -488,46 +488,53 @@ __device__ __forceinline__ CellMoments<Q, R> cell_update(R* g, bool force, R ome
     return m;
 }
 
-// D2Q9 with binary16 storage, one simulation.  The stochastic rounding turns
-// any change of a last bit into another trajectory, so the form has to be the
-// same in every kernel that may run a step: each product and sum is rounded or
-// fused as written (left to the compiler, the plain and the pipelined kernel
-// fused the rest direction differently).  rest_fused belongs to the lattice,
-// not to the launch shape: set where the pipelined kernel, which always fuses
-// the rest direction's new term, is applicable.  g may be held scaled by gscale
-// = 1 / ginv (a power of two, so exactly).  FORCE = false has the values of
-// F = 0.
-template <bool FORCE>
-__device__ __forceinline__ CellMoments<9, float> cell_update_h9(float* g, bool rest_fused, float omega,
-                                                                float Fx, float Fy, float ginv = 1.0f,
-                                                                float gscale = 1.0f)
+// Binary16 storage, one simulation, one cell at a time.  The stochastic rounding
+// turns any change of a last bit into another trajectory, so the form has to be
+// the same in every kernel that may run a step: each product and sum is rounded
+// or fused as written (left to the compiler, the plain and the pipelined kernel
+// fused the rest direction differently, and differently again after an edit).
+// rest_fused belongs to the lattice, not to the launch shape: set where the
+// pipelined kernel, which always fuses the rest direction's new term, is
+// applicable.  g may be held scaled by gscale = 1 / ginv (a power of two, so
+// exactly).  FORCE = false has the values of F = 0.
+template <int Q, bool FORCE>
+__device__ __forceinline__ CellMoments<Q, float> cell_update_h(float* g, bool rest_fused, float omega,
+                                                               float Fx, float Fy, float Fz,
+                                                               float ginv = 1.0f, float gscale = 1.0f)
 {
-    using L = Stencil<9>;
-    const CellMoments<9, float> m = cell_moments<9, float, FORCE>(g, Fx, Fy, 0.0f, ginv);
+    using L = Stencil<Q>;
+    constexpr int D = L::D;
+    const CellMoments<Q, float> m = cell_moments<Q, float, FORCE>(g, Fx, Fy, Fz, ginv);
     const float pref = __fmaf_rn(-0.5f, omega, 1.0f);
     const float om1 = __fsub_rn(1.0f, omega);
-    const float usq = __fmaf_rn(m.ux, m.ux, __fmul_rn(m.uy, m.uy));
+    float usq = __fmaf_rn(m.ux, m.ux, __fmul_rn(m.uy, m.uy));
+    if (D == 3) usq = __fmaf_rn(m.uz, m.uz, usq);
     const float dev = __fmaf_rn(-m.rho, __fmul_rn(1.5f, usq), m.drho);
     float sym0 = __fmul_rn(omega, dev);
     if constexpr (FORCE) {
-        const float uF = __fmaf_rn(m.ux, Fx, __fmul_rn(m.uy, Fy));
+        float uF = __fmaf_rn(m.ux, Fx, __fmul_rn(m.uy, Fy));
+        if (D == 3) uF = __fmaf_rn(m.uz, Fz, uF);
         sym0 = __fmaf_rn(omega, dev, -__fmul_rn(__fmul_rn(3.0f, pref), uF));
     }
     const float k2 = __fmul_rn(__fmul_rn(omega, 4.5f), m.rho);
     const float k1 = __fmul_rn(omega, m.rho);
     const float p9 = __fmul_rn(9.0f, pref);
-    const float w0 = coef_b<9, float>(0) * gscale;
-    g[0] = rest_fused ? __fmaf_rn(w0, sym0, __fmul_rn(om1, g[0])) : __fmaf_rn(om1, g[0], __fmul_rn(w0, sym0));
+    const float w0 = coef_b<Q, float>(0) * gscale;
+    // either product is rounded first (operands selected, so that no branch
+    // keeps the loads after it from being issued early)
+    const float ra = rest_fused ? w0 : om1, rb = rest_fused ? sym0 : g[0];
+    const float rc = rest_fused ? om1 : w0, rd = rest_fused ? g[0] : sym0;
+    g[0] = __fmaf_rn(ra, rb, __fmul_rn(rc, rd));
 #pragma unroll
-    for (int i = 1; i < 9; i++) {
+    for (int i = 1; i < Q; i++) {
         if (L::opp(i) < i) continue;  // each pair once
         const int o = L::opp(i);
-        const float w = coef_b<9, float>(i) * gscale;
-        const float w3 = coef_a<9, float>(i) * gscale;
-        const float cu = dot_c<9, float>(i, m.ux, m.uy, 0.0f);
+        const float w = coef_b<Q, float>(i) * gscale;
+        const float w3 = coef_a<Q, float>(i) * gscale;
+        const float cu = dot_c<Q, float>(i, m.ux, m.uy, m.uz);
         float t = __fmul_rn(k2, cu), a = __fmul_rn(k1, cu);
         if constexpr (FORCE) {
-            const float cF = dot_c<9, float>(i, Fx, Fy, 0.0f);
+            const float cF = dot_c<Q, float>(i, Fx, Fy, Fz);
             t = __fmaf_rn(k2, cu, __fmul_rn(p9, cF));
             a = __fmaf_rn(k1, cu, __fmul_rn(pref, cF));
         }

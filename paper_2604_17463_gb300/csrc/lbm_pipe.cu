@@ -377,8 +377,8 @@ k_sc_pipe(const typename StorageT<ST>::S* __restrict__ fin,
             R Fx = param_body<R>(p, 0), Fy = param_body<R>(p, 1), Fz = param_body<R>(p, 2);
             if (band) take_band_force<D, R>(F, nc, cell, Fx, Fy, Fz);
             CellMoments<Q, R> mo;
-            if constexpr (Q == 9 && ST == ST_FP16)
-                mo = cell_update_h9<true>(g, true, omega, Fx, Fy);
+            if constexpr (ST == ST_FP16)
+                mo = cell_update_h<Q, true>(g, true, omega, Fx, Fy, Fz);
             else
                 mo = cell_update<Q, R, force_mode<R, false>()>(g, band || p.has_body, omega, Fx, Fy, Fz);
             store_cell<Q, ST, false>(fout, nc, cell, g, p.scale,

@@ -72,7 +72,7 @@ __device__ __forceinline__ int bin_coord(const GridParams& g, int k, int o)
     return periodic_axis(g, k) ? wrap(o, extent(g, k)) : o + 3;
 }
 
-template <int D, typename R>
+template <int D, typename R, bool KEEP>
 __global__ void k_det_bin(const DetSlot* __restrict__ slots, const int2* __restrict__ items,
                           int nitems, int* __restrict__ bin_of, int* __restrict__ org,
                           R* __restrict__ wts, int* __restrict__ cnt, int* __restrict__ active,
@@ -96,7 +96,7 @@ __global__ void k_det_bin(const DetSlot* __restrict__ slots, const int2* __restr
         o[k] = (int)fl - 1;
         const R fr = (R)(qk - fl);  // as node_lines: FP64 split, weights in R
         R w4[4];
-        delta4_weights<D, R>(fr, w4);
+        delta4_weights<R, KEEP>(fr, w4);
         for (int s = 0; s < 4; s++) wts[(long long)it * 12 + 4 * k + s] = w4[s];
         org[3 * it + k] = o[k];
     }
@@ -429,7 +429,7 @@ k_det_gather(const DetSlot* __restrict__ slots, const int2* __restrict__ items,
     }
 }
 
-template <int D, typename R>
+template <int D, typename R, bool KEEP>
 void launch_det_t(const DetSlot* slots, const int2* items, int nitems, const DetBuffers& b,
                   int nbins, int ncelltiles, int sm_count, cudaStream_t s)
 {
@@ -437,7 +437,7 @@ void launch_det_t(const DetSlot* slots, const int2* items, int nitems, const Det
     k_det_clear<<<min((nclr + 255) / 256, 4 * sm_count), 256, 0, s>>>(b.cnt, nbins, b.active,
                                                                       ncelltiles, b.nact);
     const int nb = (nitems + 127) / 128, nb64 = (nitems + 63) / 64;
-    k_det_bin<D, R><<<nb64, 64, 0, s>>>(slots, items, nitems, b.bin_of, b.org, (R*)b.wts, b.cnt,
+    k_det_bin<D, R, KEEP><<<nb64, 64, 0, s>>>(slots, items, nitems, b.bin_of, b.org, (R*)b.wts, b.cnt,
                                        b.active, b.act_list, b.nact);
     k_det_scan<<<1, SCAN_BLOCK, 0, s>>>(b.cnt, nbins, b.start, b.cur);
     k_det_place<<<nb, 128, 0, s>>>(b.bin_of, nitems, b.cur, b.list);
@@ -454,11 +454,12 @@ void launch_spread_det(int storage, int dim, const DetSlot* slots, const int2* i
 {
     if (nitems <= 0) return;
     if (storage == ST_FP64) {
-        if (dim == 2) launch_det_t<2, double>(slots, items, nitems, b, nbins, ncelltiles, sm_count, s);
-        else launch_det_t<3, double>(slots, items, nitems, b, nbins, ncelltiles, sm_count, s);
+        if (dim == 2) launch_det_t<2, double, false>(slots, items, nitems, b, nbins, ncelltiles, sm_count, s);
+        else launch_det_t<3, double, false>(slots, items, nitems, b, nbins, ncelltiles, sm_count, s);
     } else {
-        if (dim == 2) launch_det_t<2, float>(slots, items, nitems, b, nbins, ncelltiles, sm_count, s);
-        else launch_det_t<3, float>(slots, items, nitems, b, nbins, ncelltiles, sm_count, s);
+        if (dim == 2) launch_det_t<2, float, true>(slots, items, nitems, b, nbins, ncelltiles, sm_count, s);
+        else if (keep_weights_3d(storage, true)) launch_det_t<3, float, true>(slots, items, nitems, b, nbins, ncelltiles, sm_count, s);
+        else launch_det_t<3, float, false>(slots, items, nitems, b, nbins, ncelltiles, sm_count, s);
     }
 }
 
