@@ -268,6 +268,10 @@ iblb_status iblb_step_profiled(iblb_handle h, int n_steps, double* kernel_ms);
  *   variant 3: two y-adjacent cells per thread (rows y, y + 1 of a layer)
  *              with scalar loads and stores and packed FP32x2 arithmetic
  *              (D3Q19, FP32 and binary16 storage), block_x threads per block;
+ *              in binary16, with an even nx and where no cell has a force (the
+ *              overlapped step's pass over every cell without a body force),
+ *              two such pairs per thread with 32-bit loads and stores and the
+ *              same results;
  *   variant 1: the pipelined kernel: persistent CTAs in which a producer warp
  *              stages the source rows in shared memory with bulk asynchronous
  *              copies and consumer_warps warps collide from there;

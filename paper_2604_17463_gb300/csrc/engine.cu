@@ -143,10 +143,11 @@ int regroup_kernels(const iblb_sim* h) { return use_groups(h) ? REGROUP_KERNELS 
 // The overlapped step (enqueue_step_overlapped): with an interface, and
 // (automatic mode) on a 3D lattice of at least 2^20 cells, in FP64 of at least
 // 2^15.  Below that the IB kernels of an FP32 step are too short to hide behind
-// the bulk pass and pay for the band pass: 101 x 101 x 77 50.2 us serial, 49.9
-// overlapped, 64 x 64 x 40 25.3 and 25.8; FP64 64 x 64 x 40 88.8 and 73.9,
-// 96 x 96 x 72 216 and 202, 40 x 40 x 32 71.1 and 64.3.  A 2D ring's are
-// shorter still (2048 x 512 spreading drop: 21.5 us serial, 25.5 overlapped).
+// the bulk pass and pay for the band pass: 101 x 101 x 77 49.8 us serial, 48.6
+// overlapped, 64 x 64 x 40 25.0 and 26.1; FP64 64 x 64 x 40 89.0 and 74.9,
+// 96 x 96 x 72 217 and 203, 40 x 40 x 32 71.6 and 64.5.  A 2D ring's are
+// shorter still (FP32 2048 x 512 spreading drop: 16.9 us serial, 18.9
+// overlapped).
 bool overlapped(const iblb_sim* h)
 {
     if (h->N == 0 || h->tune.step_overlap == 2) return false;
@@ -155,10 +156,15 @@ bool overlapped(const iblb_sim* h)
 }
 // The serial step of a ring with one fused IB kernel per step (k_ring);
 // the ordered spread and the overlapped step keep their separate kernels, and
-// so do calls of fewer than RING_FUSED_STEPS steps: there one launch per phase
-// and step is what a caller that checks iblb_kernel_launch_count counts on.
-// binary16 keeps them too: its stochastic rounding makes another trajectory of
-// any last bit that the order of the additions or a fused product changes.
+// so do calls of fewer than RING_FUSED_STEPS steps.  That line is not one of
+// cost: the fused step is the faster one in calls of any length (FP64 128 x 64
+// ring, us per step in calls of 1, 2, 8 and 15 steps: 21.5, 18.4, 17.2 and 16.9
+// fused, 22.5, 20.1, 19.0 and 18.9 separate).  It keeps one launch per phase and
+// step in short calls, as programs and tests that check
+// iblb_kernel_launch_count on 10 steps expect.
+// binary16 keeps the separate kernels too: its stochastic rounding makes another
+// trajectory of any last bit that the order of the additions or a fused product
+// changes.
 constexpr int RING_FUSED_STEPS = 16;
 bool ring_fused(const iblb_sim* h, int call_steps)
 {
@@ -420,17 +426,21 @@ double wetting_amplitude(const iblb_config& c)
            ((double)(c.pi_n - c.pi_m) * c.xi) * (1.0 + std::cos(th));
 }
 
-// Launch shape of a new simulation.  The pipelined kernel is the default on 3D
-// lattices of at least 2^22 cells in FP32 / binary16 (where a program that
-// cares runs the autotuner); elsewhere its few persistent CTAs cost more than
-// they hide.  Whole steps, us, pipelined against the chosen shape:
-//   D2Q9  FP64   128 x 64   22.7  18.7 (plain, 64)   2048 x 512  162  156
-//         FP32  2048 x 512  24.3  18.1 (x pairs)     512 x 128   15.6  11.2 (plain)
-//         binary16 1024 x 256  17.6  13.7 (plain)
-//   D3Q19 FP32   96 x 96 x 64  56  45 (plain, 128)   160 x 160 x 96  117  94
-//         FP64   96 x 96 x 72  640  623 (plain, 128)
-// D2Q9 FP32: x pairs need an even width and win from about 2^19 cells (1000 x
-// 250: 12.7 against 13.0 us; 512 x 128: 11.6 against 11.2).
+// Launch shape of a new simulation.  The pipelined kernel remains the default on
+// 3D lattices of at least 2^22 cells in FP32 and binary16, although its few
+// persistent CTAs cost more than they hide there too; the autotuner finds the
+// faster shape.  Whole steps, us, pipelined against the chosen shape:
+//   D2Q9  FP64   128 x 64   21.0  16.9 (plain, 64)   2048 x 512  157  150
+//         FP32  2048 x 512  23.0  16.9 (x pairs)     512 x 128   13.9  10.0 (plain)
+//         binary16 1024 x 256  19.9  16.2 (plain)
+//   D3Q19 FP32   96 x 96 x 64  52  42 (plain, 128)   160 x 160 x 96  113  78
+//         binary16 160 x 160 x 96  118  66 (plain, 128)
+//         FP64   96 x 96 x 72  234  203 (plain, 128)
+// and pipelined against the autotuner's choice from 2^22 cells:
+//         FP32  192 x 192 x 120  182  130   256 x 256 x 128  250  212
+//         binary16  the same     194  108                    252  147
+// D2Q9 FP32: x pairs need an even width and win from about 2^19 cells (2048 x
+// 512 16.9 against 19.1 us; 512 x 128 10.3 against 10.0).
 Tuning default_tuning(const iblb_sim* h)
 {
     Tuning t;

@@ -304,8 +304,9 @@ __device__ bool solve_small(int n, double* A, double* b)
 // OBS_GRID blocks: a pass's blocks each add up the previous pass's partial
 // sums for themselves.  FP64 arithmetic bounds them: in one block, on one SM's
 // pipe, the call (with the mass sum and its synchronisations) took 0.16 ms on
-// the 128 x 64 ring, 0.41 ms with 10 242 nodes and 1.63 ms with 40 962; so 0.12,
-// 0.16 and 0.79 ms.
+// the 128 x 64 ring, 0.41 ms with 10 242 nodes on 101 x 101 x 77 and 1.63 ms with
+// 40 962 on 256 x 256 x 128; with these passes and the mass sum of lbm.cu 0.10,
+// 0.14 and 0.26 ms.
 constexpr int OBS_THREADS = 256;
 constexpr int OBS_P1 = 8, OBS_P2 = 20, OBS_P3 = 2;  // doubles per block and pass
 
@@ -523,7 +524,7 @@ __global__ void __launch_bounds__(32) k_obs_last(ObsArgs a, int grid)
 // The central second moments in the shear plane (x and the wall axis) give
 // the semi-axes sqrt(4 lambda / area) (2D) or sqrt(5 lambda / volume) (3D).
 // Three kernels: node sums, simplex sums about their mean, results; up to
-// OBS_GRID blocks (the call with 20 480 faces took 0.49 ms in one block, so 0.06).
+// OBS_GRID blocks (the call with 20 480 faces took 0.49 ms in one block, with 81 920 now 0.07).
 __global__ void __launch_bounds__(OBS_THREADS) k_def_mean(int dim, const double* __restrict__ q, int N, double* part)
 {
     __shared__ double sh[3][OBS_THREADS / 32];

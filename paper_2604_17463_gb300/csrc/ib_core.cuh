@@ -427,7 +427,7 @@ __device__ __forceinline__ void ring_node_force(const double* __restrict__ q, in
 // through memory: interpolation, forces and spread of a ring are one kernel
 // instead of three.  The positions go to a second array (the neighbours'
 // warps read the first).  Step of the FP64 128 x 64 ring (213 nodes) 18.7 ->
-// 16.7 us, of the FP32 2048 x 512 one (2000 nodes) 18.1 -> 16.6 us.
+// 16.9 us, of the FP32 2048 x 512 one (2000 nodes) 18.1 -> 16.9 us.
 constexpr int RING_OWN = 30;
 
 template <typename R, bool FIRST>

@@ -369,7 +369,9 @@ __device__ __forceinline__ CellMoments<Q, R> cell_moments(const R* g, R Fx, R Fy
 //
 // FORCE = false drops every term in F: the kernels take it for the cells
 // outside the band when there is no body force, 97 % of a 3D drop's lattice.
-// Its values are those of FORCE = true with F = 0, bit for bit.
+// Its values are those of FORCE = true with F = 0: bit for bit in FP64 and in the
+// paired and binary16 forms, where every rounding is written out, and as far as
+// the compiler fuses both alike in scalar FP32.
 // In FP64 the weights are multiplied into the cell's coefficients once per
 // speed class instead of once per direction: FP64 arithmetic bounds those
 // kernels (a warp instruction holds the SM's pipe for 16 clocks).  FP32 keeps
