@@ -29,7 +29,8 @@
 // index work of a node, and most of the step.  10 242 nodes on 96 x 96 x 72 in
 // FP64: spread 447 -> 93 us per step (128 before the bins were sorted by warps).
 // Only the order of the additions differs from the scatter: the weights are
-// the same numbers, formed the same way.  The same kernels serve the
+// the same numbers, formed the same way (3D binary16: to their last bits, see
+// delta4_weights).  The same kernels serve the
 // single-simulation engine (one slot, node item = node id) and the batched
 // engine (items = (slot, node) pairs in slot order, bins and cell tiles
 // numbered globally across slots).
